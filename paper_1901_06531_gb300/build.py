@@ -25,7 +25,8 @@ LIB_DEBUG = os.path.join(HERE, "libmixfft_debug.so")
 # graph (MF_TRACE, read back with mf_trace_read)
 BUILD_TRACE = os.path.join(HERE, "_build_trace")
 LIB_TRACE = os.path.join(HERE, "libmixfft_trace.so")
-SOURCES = ["transform.cu", "transform2_f32.cu", "transform2_f64.cu", "pointwise.cu", "cg.cu", "history.cu",
+SOURCES = ["transform.cu", "transform2_f32.cu", "transform2_f64.cu", "transformg_f32.cu",
+           "transformg_f64.cu", "pointwise.cu", "cg.cu", "history.cu",
            "mixfft.cu", "noalloc.cu", "cufft_path.cu", "adjoint.cu", "transform2_dw.cu",
            "constitutive_dw.cu", "probe.cu"]
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]

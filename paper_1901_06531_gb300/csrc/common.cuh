@@ -1,7 +1,7 @@
-// Shared device machinery: complex helpers, per-axis FFT plans and the
-// in-place shared-memory FFT stages used by every transform kernel.
+// Shared device machinery: complex helpers, per-axis FFT plans, small DFTs
+// and the scalar blocks of the solvers.
 //
-// Transforms are computed in place with mixed-radix (2, 3, 4) stages.  The
+// Transforms are computed in place with mixed-radix stages.  The
 // forward transform is decimation in frequency (natural order in, digit-
 // reversed order out), the inverse is its exact adjoint, decimation in time
 // (digit-reversed in, natural out).  The spectrum therefore never needs a
@@ -12,7 +12,7 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
-#define MF_MAX_STAGES 10
+#define MF_MAX_STAGES 3
 
 // Bounds checks of the debug build (compiled with -DMF_DEBUG; release builds
 // compile them away).  MF_AT(i, n) is i when 0 <= i < n; otherwise the
@@ -67,10 +67,28 @@ inline int stride_grid(long long n, int threads = 256) {
   return (int)(b < 1 ? 1 : (b < 152 * 8 ? b : 152 * 8));
 }
 
+// Quotients by a run-time divisor d through m = ceil(2^32 / d) (d > 1).
+struct FastDiv {
+  int d;
+  unsigned m;
+};
+inline FastDiv fast_div(int d) {
+  FastDiv f;
+  f.d = d;
+  f.m = d > 1 ? (unsigned)((0x100000000ull + (unsigned)d - 1) / (unsigned)d) : 0u;
+  return f;
+}
+
+// Stages of a transform in decimation-in-frequency order (built by plan.h).
 struct AxisPlan {
-  int n;                     // transform length
-  int nst;                   // number of stages
-  int rad[MF_MAX_STAGES];    // radix of each stage in DIF order
+  int n;                        // transform length
+  int nst;                      // number of stages
+  int ntab;                     // length of the twiddle table, a multiple of n
+  int rad[MF_MAX_STAGES];       // radix
+  int m[MF_MAX_STAGES];         // sub-transform length / radix
+  int tstep[MF_MAX_STAGES];     // twiddle table step
+  FastDiv dm[MF_MAX_STAGES];    // by m
+  FastDiv nb[MF_MAX_STAGES];    // by the butterflies of a sequence, n / radix
 };
 
 template <typename T> struct CT;
@@ -155,78 +173,6 @@ template <bool INV, typename C> struct Radix<3, INV, C> {
     v[2] = csub(t2, it3);
   }
 };
-
-// One in-place radix-R stage over `nseq` sequences of length n in shared
-// memory.  Element j of sequence s is at buf[(s / nlo) * hs + (s % nlo) * ls + j * es].
-// L is the current sub-transform length (n at the first DIF stage); the
-// twiddle table holds W_ntab^t = exp(-2 pi i t / ntab) with n | ntab.
-// SEQ_FAST chooses the thread order: consecutive threads walk sequences
-// (strided transforms) or butterflies (contiguous transforms).
-template <typename C, int R, bool INV, bool SEQ_FAST>
-__device__ __forceinline__ void fft_stage(C* buf, int n, int L, int nseq, int nlo, int hs,
-                                          int ls, int es, const C* tw, int ntab, int ext) {
-  const int m = L / R;
-  const int nb = n / R;
-  const int total = nb * nseq;
-  const int tstep = ntab / L;
-  for (int t = threadIdx.x; t < total; t += blockDim.x) {
-    int s, b;
-    if (SEQ_FAST) { s = t % nseq; b = t / nseq; } else { b = t % nb; s = t / nb; }
-    const int blk = b / m;
-    const int j0 = b - blk * m;
-    const int base = (s / nlo) * hs + (s % nlo) * ls + (blk * L + j0) * es;
-    const int step = m * es;
-    C v[R];
-#pragma unroll
-    for (int r = 0; r < R; ++r) v[r] = buf[MF_AT(base + r * step, ext)];
-    if (!INV) {
-      Radix<R, false, C>::run(v);
-#pragma unroll
-      for (int k = 1; k < R; ++k) v[k] = cmul(v[k], tw[MF_AT(j0 * k * tstep, ntab)]);
-    } else {
-#pragma unroll
-      for (int k = 1; k < R; ++k) v[k] = cmulc(v[k], tw[MF_AT(j0 * k * tstep, ntab)]);
-      Radix<R, true, C>::run(v);
-    }
-#pragma unroll
-    for (int r = 0; r < R; ++r) buf[MF_AT(base + r * step, ext)] = v[r];
-  }
-}
-
-template <typename C, bool INV, bool SEQ_FAST>
-__device__ __forceinline__ void fft_stage_dispatch(int R, C* buf, int n, int L, int nseq, int nlo,
-                                                   int hs, int ls, int es, const C* tw, int ntab, int ext) {
-  if (R == 4) fft_stage<C, 4, INV, SEQ_FAST>(buf, n, L, nseq, nlo, hs, ls, es, tw, ntab, ext);
-  else if (R == 2) fft_stage<C, 2, INV, SEQ_FAST>(buf, n, L, nseq, nlo, hs, ls, es, tw, ntab, ext);
-  else fft_stage<C, 3, INV, SEQ_FAST>(buf, n, L, nseq, nlo, hs, ls, es, tw, ntab, ext);
-}
-
-// Full transform of every sequence: DIF forward (INV = false) or its adjoint
-// DIT inverse (INV = true, unnormalised).  Ends with __syncthreads(); the
-// caller synchronises before the first stage.  ext: elements of buf (the
-// debug build checks every index against it).
-template <typename C, bool INV, bool SEQ_FAST>
-__device__ __forceinline__ void fft_run(C* buf, const AxisPlan& pl, int nseq, int nlo, int hs,
-                                        int ls, int es, const C* tw, int ntab, int ext) {
-  if (!INV) {
-    int L = pl.n;
-    for (int st = 0; st < pl.nst; ++st) {
-      const int R = pl.rad[st];
-      fft_stage_dispatch<C, false, SEQ_FAST>(R, buf, pl.n, L, nseq, nlo, hs, ls, es, tw, ntab, ext);
-      L /= R;
-      __syncthreads();
-    }
-  } else {
-    int Ls[MF_MAX_STAGES];
-    int L = pl.n;
-    for (int st = 0; st < pl.nst; ++st) { Ls[st] = L; L /= pl.rad[st]; }
-    for (int st = pl.nst - 1; st >= 0; --st) {
-      fft_stage_dispatch<C, true, SEQ_FAST>(pl.rad[st], buf, pl.n, Ls[st], nseq, nlo, hs, ls, es,
-                                            tw, ntab, ext);
-      __syncthreads();
-    }
-  }
-}
 
 // Index of the packed symmetric 9x9 tangent entry (a, b), a, b in [0, 9).
 __host__ __device__ __forceinline__ int sym45(int a, int b) {

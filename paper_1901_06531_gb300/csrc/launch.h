@@ -29,37 +29,38 @@ cudaError_t launch_k(bool pdl, void (*k)(KArgs...), dim3 g, dim3 b, size_t sm, c
 }
 
 struct XYArgs {
-  int v2;          // 1: fixed-size kernels (transform2*.cu), tables of that layout
+  int v2;          // 1: fixed-size kernels (transform2*.cu), tables of that layout; 0: any-size (transformg.cuh)
   int split;       // with v2: separate row (x) and column (y) kernels (transform3.cuh)
   const int* skip; // if non-null and *skip != 0 the kernel returns at once (finished CG)
-  int fin;         // fused (v2, not split) inverse pass with the CG update: finish beta in its last block
-  int pdl;         // v2 fused kernels: launch with programmatic dependent launch (see launch_k)
+  int fin;         // fused (not split) inverse pass with the CG update: finish beta in its last block
+  int pdl;         // fused kernels: launch with programmatic dependent launch (see launch_k)
   int persist;     // FP32 v2 forward pass as the persistent bulk-copy kernel (k_xyf_p)
   int cluster_f;   // FP32 v2 forward pass (nx = 128) as the two-CTA cluster kernel (k_xyf_c)
   int cluster_i;   // FP32 v2 inverse pass (nx = 128) as the two-CTA cluster kernel (k_xyi_c)
   int* flags;      // device flags word (MF_FLAG_TIMEOUT from bounded waits), or null
   int nx, ny, nz;
   long long N;
-  AxisPlan px;     // length nx
-  AxisPlan pyh;    // length ny/2 (the y transform after its first radix-2 stage)
+  AxisPlan px;     // any-size kernels: half-length x transform (nx / 2, table W_nx) and y transform
+  AxisPlan py;
+  FastDiv dny, dh; // any-size kernels: by ny, by nx / 2
   const void* twx; // W_nx^t, t < nx   (complex of the kernel's type)
   const void* twy; // W_ny^t, t < ny
-  const int* xpos; // position of x-frequency k after the x DIF, k < nx
+  const int* xpos; // slot of x-frequency k, k < nx / 2
 };
 
 struct ZArgs {
-  int v2;
+  int v2;            // 1: fixed-size kernels; 0: any-size
   const int* skip;
-  int pdl;           // v2 kernels: launch with programmatic dependent launch (see launch_k)
+  int pdl;           // launch with programmatic dependent launch (see launch_k)
   int nx, ny, nz;
   long long N;
-  AxisPlan pz;
+  AxisPlan pz;       // any-size kernels
+  FastDiv dh, dseq;  // any-size kernels: by nx / 2, by the sequences of a block (set by the launcher)
   const void* twz;   // W_nz^t
   const int* xk;     // slot -> kx
-  const int* xe;     // slot -> parity e
-  const int* yk;     // row q' -> ky half index
+  const int* yk;     // row -> ky
   const int* zk;     // position -> kz
-  int S;             // columns per block
+  int S;             // columns per block (fixed-size kernels)
   unsigned mask;     // bit c set: component c stress controlled
   double scale;      // multiplies every coefficient (1/N, or -1/N for the residual)
   double add[9];     // added at the null frequency after scaling (residual: P-bar)
@@ -72,11 +73,15 @@ struct ZArgs {
 // Process-wide count of kernel launches issued by the library.
 extern long long g_mf_launches;
 
-// transform2_f32.cu / transform2_f64.cu: fixed-size kernels for square x-y
-// planes nx = ny and nx, nz in {16, 32, 48, 64, 96, 128}.  Their spectrum layout:
-// per (c, z) ny rows (digit-reversed ky, yk table of ny entries) of nx/2 slots
-// (digit-reversed kx, xk table of nx/2 entries), xpos = slot of kx.
-bool mf_v2_supported(int nx, int ny, int nz);
+// Spectrum layout of all transform kernels: per (c, z) ny rows
+// (digit-reversed ky, yk table of ny entries) of nx/2 slots (digit-reversed
+// kx, xk table of nx/2 entries), xpos = slot of kx.
+// transform2_f32.cu / transform2_f64.cu: fixed-size kernels, the x-y passes
+// for square planes nx = ny in {16, 32, 48, 64, 96, 128} (256: split), the
+// z-pass for nz in {16, 32, 48, 64, 96, 128, 256}.
+bool mf_v2_supported(int nx, int ny, int nz);   // all three axes
+bool mf_v2_xy(int nx, int ny);                  // the fused x-y passes
+bool mf_v2_z(int nx, int ny, int nz);           // the z-pass (whole tiles of columns)
 // the split row/column x-y kernels exist for these plane sizes (nx = ny)
 bool mf_split_supported(int nx);
 // the persistent FP32 forward kernel exists for these plane sizes (nx = ny)
@@ -95,6 +100,16 @@ cudaError_t mf_v2_xyi_f64(int mode, const void* spec, void* out, double* partial
                           const Scalars* sc, cudaStream_t st);
 cudaError_t mf_v2_zp_f64(int mode, void* spec, const ZArgs& a, cudaStream_t st);
 
+// transformg_f32.cu / transformg_f64.cu: any-size kernels (modes as above)
+cudaError_t mf_g_xyf_f32(const void* in, void* spec, const XYArgs& a, cudaStream_t st);
+cudaError_t mf_g_xyi_f32(int mode, const void* spec, void* out, double* partials, const XYArgs& a,
+                         const Scalars* sc, cudaStream_t st);
+cudaError_t mf_g_zp_f32(int mode, void* spec, const ZArgs& a, cudaStream_t st);
+cudaError_t mf_g_xyf_f64(const void* in, void* spec, const XYArgs& a, cudaStream_t st);
+cudaError_t mf_g_xyi_f64(int mode, const void* spec, void* out, double* partials, const XYArgs& a,
+                         const Scalars* sc, cudaStream_t st);
+cudaError_t mf_g_zp_f64(int mode, void* spec, const ZArgs& a, cudaStream_t st);
+
 // transform2_f32.cu: one block waits, at most max_polls polls, on a barrier
 // nothing arrives at, and sets MF_FLAG_TIMEOUT in *flags (device int)
 cudaError_t mf_launch_wait_selftest(int max_polls, int* flags, cudaStream_t st);
@@ -108,8 +123,6 @@ cudaError_t mf_v2_xyi_dw(const void* spec, double* out, double* partials, const 
 // transform.cu
 // b = -G*(P - P-bar) (null frequency per za); dw: double-word transforms
 // (fixed-size kernels only; xa, za then point at the double-word tables).
-// The generic kernels also leave block partial sums of b.b in partials; the
-// fixed-size ones do not (nothing reads them).
 cudaError_t mf_launch_residual(const double* P, void* spec, double* b, double* partials,
                                const XYArgs& xa, const ZArgs& za, bool dw, cudaStream_t st);
 // The same residual with FP32 transforms (fixed-size kernels; xa, za with the

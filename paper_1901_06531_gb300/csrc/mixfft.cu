@@ -16,6 +16,7 @@
 #include "dw.cuh"
 #include "fft2.cuh"
 #include "launch.h"
+#include "plan.h"
 #include "predict.cuh"
 
 namespace {
@@ -45,39 +46,6 @@ void trace_mark(cudaStream_t, int) {}
 
 constexpr int kMaxPhases = 65536;
 constexpr int kPointwiseBlocks = 152 * 8;
-
-bool make_plan(int n, AxisPlan* p) {
-  p->n = n;
-  p->nst = 0;
-  int m = n;
-  while (m % 4 == 0) { p->rad[p->nst++] = 4; m /= 4; }
-  if (m % 2 == 0) { p->rad[p->nst++] = 2; m /= 2; }
-  while (m % 3 == 0) {
-    if (p->nst >= MF_MAX_STAGES) return false;
-    p->rad[p->nst++] = 3;
-    m /= 3;
-  }
-  return m == 1 && p->nst <= MF_MAX_STAGES;
-}
-
-// Position of frequency k after the DIF stages of plan p.
-int dif_pos(const AxisPlan& p, int k) {
-  int pos = 0, L = p.n;
-  for (int st = 0; st < p.nst; ++st) {
-    const int r = p.rad[st], m = L / r;
-    pos += m * (k % r);
-    k /= r;
-    L = m;
-  }
-  return pos;
-}
-
-bool smooth_size(int n) {
-  if (n < 1) return false;
-  while (n % 2 == 0) n /= 2;
-  while (n % 3 == 0) n /= 3;
-  return n == 1;
-}
 
 size_t align256(size_t x) { return (x + 255) & ~(size_t)255; }
 
@@ -252,10 +220,11 @@ struct mf_ctx {
   int nx, ny, nz;
   long long N;
   int prec;
-  int v2 = 0;              // fixed-size transform kernels and their table layout
+  int v2 = 0;              // fixed-size transform kernels on all three axes
+  int v2xy = 0, v2z = 0;   // fixed-size x-y passes, z-pass (else the any-size kernels)
   int xy_split = 0;        // with v2: separate row and column kernels for the x-y transform
   cudaStream_t st;
-  AxisPlan px, pyh, pz;
+  AxisPlan px, py, pz;     // any-size kernels: nx / 2, ny, nz
   int zS;                  // z-pass tile of the operator (CG loop)
   int zSr = 8;             // z-pass tile of the residual (fixed-size kernels)
   // workspace
@@ -263,7 +232,7 @@ struct mf_ctx {
   size_t ws_need = 0;
   // offsets into the workspace
   size_t oF, oP, ob, oK, ox, or_, op, op2, oAp, oH, ospec, ophase, oscale, oscale32, otable,
-      otable32, otabledw, opart, osc, ores, oxpos, oxk, oxe, oyk, ozk, otw64, otw32, otwdw;
+      otable32, otabledw, opart, osc, ores, oxpos, oxk, oyk, ozk, otw64, otw32, otwdw;
   // load-history state and tables (history.cu)
   size_t ohist, othout, othin, oFprev, oFprev2;
   int predictor = MF_PRED_UNIFORM;  // mf_set_predictor
@@ -326,20 +295,21 @@ size_t tw_offset(const mf_ctx* c, bool f32, bool dw, size_t* esz) {
 
 XYArgs xy_args(const mf_ctx* c, bool f32, bool dw = false) {
   XYArgs a{};
-  a.v2 = c->v2;
+  a.v2 = c->v2xy;
   a.split = c->xy_split;
   a.skip = nullptr;
   a.fin = 0;
-  // the fused fixed-size kernels wait for their predecessor themselves
-  // (pdl_wait): launch them with programmatic dependent launch everywhere
-  a.pdl = (c->v2 && !c->xy_split) ? 1 : 0;
+  // the fused kernels wait for their predecessor themselves (pdl_wait):
+  // launch them with programmatic dependent launch everywhere
+  a.pdl = c->xy_split ? 0 : 1;
   a.persist = (f32 && !dw && c->xy_persist && c->v2 && !c->xy_split) ? 1 : 0;
   const bool clu = f32 && !dw && c->v2 && !c->xy_split && mf_cluster_supported(c->nx);
   a.cluster_f = (clu && (c->xy_cluster & 1)) ? 1 : 0;
   a.cluster_i = (clu && (c->xy_cluster & 2)) ? 1 : 0;
   a.flags = &c->at<Scalars>(c->osc)->flags;
   a.nx = c->nx; a.ny = c->ny; a.nz = c->nz; a.N = c->N;
-  a.px = c->px; a.pyh = c->pyh;
+  a.px = c->px; a.py = c->py;
+  a.dny = fast_div(c->ny); a.dh = fast_div(c->nx / 2);
   size_t esz;
   const size_t tw = tw_offset(c, f32, dw, &esz);
   a.twx = c->ws + tw;
@@ -351,15 +321,15 @@ XYArgs xy_args(const mf_ctx* c, bool f32, bool dw = false) {
 ZArgs z_args(const mf_ctx* c, bool f32, const uint8_t* mask, double scale, bool dw = false) {
   ZArgs a{};
   memset(&a, 0, sizeof(a));
-  a.v2 = c->v2;
-  a.pdl = c->v2;   // the fixed-size z-pass waits for its predecessor itself
+  a.v2 = c->v2z;
+  a.pdl = 1;   // the z-pass waits for its predecessor itself
   a.nx = c->nx; a.ny = c->ny; a.nz = c->nz; a.N = c->N;
   a.pz = c->pz;
+  a.dh = fast_div(c->nx / 2);
   size_t esz;
   const size_t tw = tw_offset(c, f32, dw, &esz);
   a.twz = c->ws + tw + esz * (c->nx + c->ny);
   a.xk = c->at<int>(c->oxk);
-  a.xe = c->at<int>(c->oxe);
   a.yk = c->at<int>(c->oyk);
   a.zk = c->at<int>(c->ozk);
   a.S = c->zS;
@@ -536,15 +506,15 @@ cudaError_t capture_cg_body(mf_ctx* c, cudaStream_t cs, cudaGraph_t body, const 
     za.lin = sc->lin;
     za.lin_alpha = &sc->alpha;
   }
-  // the fused x-y inverse kernel finishes beta itself; the split and generic
-  // kernels leave it to k_fin_beta
-  xa.fin = (xa.v2 && !xa.split) ? 1 : 0;
+  // the fused x-y inverse kernels finish beta themselves; the split ones
+  // leave it to k_fin_beta
+  xa.fin = xa.split ? 0 : 1;
   // programmatic dependent launch along the body (tangent, the fused
   // transform passes, the loop condition): each kernel is scheduled as its
   // predecessor's blocks exit, loads its constant tables, then waits for the
   // predecessor's completion (saves the launch gap: 8 CG-bound 32^3 cells
   // solve in half the time; neutral at 128^3)
-  const bool pdl = xa.v2 && !xa.split;
+  const bool pdl = !xa.split;
   const TangentArgs ta = tangent_args(c);
   const int tk = tangent_kind(c);
   const int nplanes = mf_xy_blocks(c->ny, c->nz, c->xy_split != 0);
@@ -557,7 +527,7 @@ cudaError_t capture_cg_body(mf_ctx* c, cudaStream_t cs, cudaGraph_t body, const 
   }
   // per iteration: tangent, the transform passes (two more for the split x-y
   // kernels), k_fin_beta unless fused; k_cg_cond once per body
-  c->cg_body_kernels = 2 * (1 + ((xa.v2 && xa.split) ? 5 : 3) + (xa.fin ? 0 : 1)) + 1;
+  c->cg_body_kernels = 2 * (1 + (xa.split ? 5 : 3) + (xa.fin ? 0 : 1)) + 1;
   if (e == cudaSuccess) e = mf_launch_cg_cond(sc, h, cs, pdl);
   cudaGraph_t captured = nullptr;
   const cudaError_t e2 = cudaStreamEndCapture(cs, &captured);
@@ -1311,7 +1281,7 @@ int mf_create(mf_ctx** out, int nx, int ny, int nz, int precision, void* stream)
   *out = nullptr;
   if (precision != MF_FP64 && precision != MF_FP32_INNER) return MF_INVALID_ARG;
   if (nx < 4 || ny < 4 || nz < 2 || nx > 256 || ny > 256 || nz > 256) return MF_INVALID_ARG;
-  if ((nx & 1) || (ny & 1) || !smooth_size(nx) || !smooth_size(ny) || !smooth_size(nz))
+  if ((nx & 1) || (ny & 1) || !mf_smooth_size(nx) || !mf_smooth_size(ny) || !mf_smooth_size(nz))
     return MF_INVALID_ARG;
   // one component's x-y plane must fit in shared memory (FP64 residual),
   // unless the split row/column kernels serve the plane
@@ -1325,16 +1295,15 @@ int mf_create(mf_ctx** out, int nx, int ny, int nz, int precision, void* stream)
   c->serial = ++g_ctx_serial;
   memset(&c->keep, 0, sizeof(c->keep));
   c->v2 = mf_v2_supported(nx, ny, nz) ? 1 : 0;
+  c->v2xy = (c->v2 || mf_v2_xy(nx, ny)) ? 1 : 0;
+  c->v2z = mf_v2_z(nx, ny, nz) ? 1 : 0;
   c->xy_split = big_plane ? 1 : 0;
   c->st = (cudaStream_t)stream;
-  if (!make_plan(nx, &c->px) || !make_plan(ny / 2, &c->pyh) || !make_plan(nz, &c->pz)) {
+  if (!mf_make_plan(nx / 2, nx, &c->px) || !mf_make_plan(ny, ny, &c->py) || !mf_make_plan(nz, nz, &c->pz)) {
     delete c;
     return MF_INVALID_ARG;
   }
-  // z-pass tile: columns per block so that 9 * nz * S complex doubles fit
-  int S = 16;
-  while (S > 1 && (size_t)9 * nz * S * sizeof(double2) > 150 * 1024) S /= 2;
-  c->zS = S;
+  c->zS = 8;   // until the autotuner chooses
   // pointwise passes: one voxel per thread for small cells, else 8 blocks per SM
   c->pw_blocks = (int)((c->N + 255) / 256 < kPointwiseBlocks ? (c->N + 255) / 256 : kPointwiseBlocks);
 
@@ -1371,7 +1340,6 @@ int mf_create(mf_ctx** out, int nx, int ny, int nz, int precision, void* stream)
   c->ores = take(9 * sizeof(double));
   c->oxpos = take(nx * sizeof(int));
   c->oxk = take(nx * sizeof(int));
-  c->oxe = take(nx * sizeof(int));
   c->oyk = take(ny * sizeof(int));
   c->ozk = take(nz * sizeof(int));
   c->otw64 = take((nx + ny + nz) * sizeof(double2));
@@ -1392,25 +1360,14 @@ int mf_bind_workspace(mf_ctx* c, void* dev, size_t bytes) {
   free_cg_graph(c);
   // host-built tables: digit-reversal maps and twiddles
   const int nx = c->nx, ny = c->ny, nz = c->nz;
-  std::vector<int> xpos(nx, 0), xk(nx, 0), xe(nx, 0), yk(ny, 0), zk(nz, 0);
-  if (c->v2) {
-    // half-length rows: slot of kx < nx/2; rows hold ky in digit-reversed order
-    const int h = nx / 2;
-    for (int k = 0; k < h; ++k) xpos[k] = fft2::dif_pos(h, k);
-    for (int k = 0; k < h; ++k) xk[xpos[k]] = k;
-    for (int k = 0; k < ny; ++k) yk[fft2::dif_pos(ny, k)] = k;
-    for (int k = 0; k < nz; ++k) zk[fft2::dif_pos(nz, k)] = k;
-  } else {
-    for (int k = 0; k < nx; ++k) xpos[k] = dif_pos(c->px, k);
-    for (int k = 0; k < nx; ++k) {
-      const int s = xpos[k];
-      if (k < nx / 2) { xk[s] = k; xe[s] = 0; }
-      else if (k == nx / 2) { xk[s] = 0; xe[s] = 1; }
-      else { xk[s] = nx - k; xe[s] = 1; }
-    }
-    for (int k = 0; k < ny / 2; ++k) yk[dif_pos(c->pyh, k)] = k;
-    for (int k = 0; k < nz; ++k) zk[dif_pos(c->pz, k)] = k;
-  }
+  std::vector<int> xpos(nx, 0), xk(nx, 0), yk(ny, 0), zk(nz, 0);
+  // half-length rows: slot of kx < nx/2; rows hold ky, planes kz in
+  // digit-reversed order of the kernels that serve the axis
+  const int h = nx / 2;
+  for (int k = 0; k < h; ++k) xpos[k] = c->v2xy ? fft2::dif_pos(h, k) : mf_plan_pos(c->px, k);
+  for (int k = 0; k < h; ++k) xk[xpos[k]] = k;
+  for (int k = 0; k < ny; ++k) yk[c->v2xy ? fft2::dif_pos(ny, k) : mf_plan_pos(c->py, k)] = k;
+  for (int k = 0; k < nz; ++k) zk[c->v2z ? fft2::dif_pos(nz, k) : mf_plan_pos(c->pz, k)] = k;
   std::vector<double2> tw64(nx + ny + nz);
   std::vector<float2> tw32(nx + ny + nz);
   std::vector<dwc> twdw(nx + ny + nz);
@@ -1431,7 +1388,6 @@ int mf_bind_workspace(mf_ctx* c, void* dev, size_t bytes) {
   };
   put(c->oxpos, xpos.data(), nx * sizeof(int));
   put(c->oxk, xk.data(), nx * sizeof(int));
-  put(c->oxe, xe.data(), nx * sizeof(int));
   put(c->oyk, yk.data(), ny * sizeof(int));
   put(c->ozk, zk.data(), nz * sizeof(int));
   put(c->otw64, tw64.data(), tw64.size() * sizeof(double2));

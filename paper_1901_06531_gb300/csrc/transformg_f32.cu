@@ -1,0 +1,13 @@
+// FP32 instances of the any-size transform kernels.
+#include "transformg.cuh"
+
+cudaError_t mf_g_xyf_f32(const void* in, void* spec, const XYArgs& a, cudaStream_t st) {
+  return trg::xyf<float>(in, spec, a, st);
+}
+cudaError_t mf_g_xyi_f32(int mode, const void* spec, void* out, double* partials, const XYArgs& a,
+                         const Scalars* sc, cudaStream_t st) {
+  return trg::xyi<float>(mode, spec, out, partials, a, sc, st);
+}
+cudaError_t mf_g_zp_f32(int mode, void* spec, const ZArgs& a, cudaStream_t st) {
+  return trg::zp<float>(mode, spec, a, st);
+}

@@ -12,7 +12,8 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
-#define MF_MAX_STAGES 3
+#define MF_MAX_STAGES 10
+#define MF_MAX_PASSES 4
 
 // Bounds checks of the debug build (compiled with -DMF_DEBUG; release builds
 // compile them away).  MF_AT(i, n) is i when 0 <= i < n; otherwise the
@@ -79,16 +80,23 @@ inline FastDiv fast_div(int d) {
   return f;
 }
 
-// Stages of a transform in decimation-in-frequency order (built by plan.h).
+// One pass of an any-size transform over memory: a stage of radix r1 and, with
+// r2 > 1, the stage of radix r2 after it.
+struct AxisPass {
+  int r1, r2;
+  int tstep1, tstep2;   // twiddle table steps of the two stages
+  FastDiv dm;           // by the last stage's sub-transform length / radix
+  FastDiv nb;           // by the butterflies of a sequence, n / (r1 r2)
+};
+
+// Stages of a transform in decimation-in-frequency order (built by plan.h)
+// and their grouping into passes.
 struct AxisPlan {
   int n;                        // transform length
-  int nst;                      // number of stages
   int ntab;                     // length of the twiddle table, a multiple of n
-  int rad[MF_MAX_STAGES];       // radix
-  int m[MF_MAX_STAGES];         // sub-transform length / radix
-  int tstep[MF_MAX_STAGES];     // twiddle table step
-  FastDiv dm[MF_MAX_STAGES];    // by m
-  FastDiv nb[MF_MAX_STAGES];    // by the butterflies of a sequence, n / radix
+  int nst, npass;
+  unsigned char rad[MF_MAX_STAGES];
+  AxisPass pass[MF_MAX_PASSES];
 };
 
 template <typename T> struct CT;

@@ -40,25 +40,26 @@ struct XYArgs {
   int* flags;      // device flags word (MF_FLAG_TIMEOUT from bounded waits), or null
   int nx, ny, nz;
   long long N;
-  AxisPlan px;     // any-size kernels: half-length x transform (nx / 2, table W_nx) and y transform
-  AxisPlan py;
-  FastDiv dny, dh; // any-size kernels: by ny, by nx / 2
+  AxisPlan px;     // any-size kernels: length nx
+  AxisPlan py;     // any-size kernels: length ny / 2 (the y transform after its first radix-2 stage)
+  FastDiv dhy, dnx;   // any-size kernels: by ny / 2, by nx
   const void* twx; // W_nx^t, t < nx   (complex of the kernel's type)
   const void* twy; // W_ny^t, t < ny
-  const int* xpos; // slot of x-frequency k, k < nx / 2
+  const int* xpos; // slot of x-frequency k (any-size kernels: k < nx, fixed-size: k < nx / 2)
 };
 
 struct ZArgs {
-  int v2;            // 1: fixed-size kernels; 0: any-size
+  int v2;            // 1: fixed-size kernels (transform2*.cu); 0: any-size (transformg.cuh)
   const int* skip;
   int pdl;           // launch with programmatic dependent launch (see launch_k)
   int nx, ny, nz;
   long long N;
   AxisPlan pz;       // any-size kernels
-  FastDiv dh, dseq;  // any-size kernels: by nx / 2, by the sequences of a block (set by the launcher)
+  FastDiv dnx, dseq; // any-size kernels: by nx, by the sequences of a block (set by the launcher)
   const void* twz;   // W_nz^t
   const int* xk;     // slot -> kx
-  const int* yk;     // row -> ky
+  const int* xe;     // any-size kernels: slot -> parity e
+  const int* yk;     // row -> ky (any-size kernels: ky = 2 yk + e)
   const int* zk;     // position -> kz
   int S;             // columns per block (fixed-size kernels)
   unsigned mask;     // bit c set: component c stress controlled
@@ -73,15 +74,11 @@ struct ZArgs {
 // Process-wide count of kernel launches issued by the library.
 extern long long g_mf_launches;
 
-// Spectrum layout of all transform kernels: per (c, z) ny rows
-// (digit-reversed ky, yk table of ny entries) of nx/2 slots (digit-reversed
-// kx, xk table of nx/2 entries), xpos = slot of kx.
-// transform2_f32.cu / transform2_f64.cu: fixed-size kernels, the x-y passes
-// for square planes nx = ny in {16, 32, 48, 64, 96, 128} (256: split), the
-// z-pass for nz in {16, 32, 48, 64, 96, 128, 256}.
-bool mf_v2_supported(int nx, int ny, int nz);   // all three axes
-bool mf_v2_xy(int nx, int ny);                  // the fused x-y passes
-bool mf_v2_z(int nx, int ny, int nz);           // the z-pass (whole tiles of columns)
+// transform2_f32.cu / transform2_f64.cu: fixed-size kernels for square x-y
+// planes nx = ny and nx, nz in {16, 32, 48, 64, 96, 128}.  Their spectrum layout:
+// per (c, z) ny rows (digit-reversed ky, yk table of ny entries) of nx/2 slots
+// (digit-reversed kx, xk table of nx/2 entries), xpos = slot of kx.
+bool mf_v2_supported(int nx, int ny, int nz);
 // the split row/column x-y kernels exist for these plane sizes (nx = ny)
 bool mf_split_supported(int nx);
 // the persistent FP32 forward kernel exists for these plane sizes (nx = ny)

@@ -220,11 +220,10 @@ struct mf_ctx {
   int nx, ny, nz;
   long long N;
   int prec;
-  int v2 = 0;              // fixed-size transform kernels on all three axes
-  int v2xy = 0, v2z = 0;   // fixed-size x-y passes, z-pass (else the any-size kernels)
+  int v2 = 0;              // fixed-size transform kernels and their table layout
   int xy_split = 0;        // with v2: separate row and column kernels for the x-y transform
   cudaStream_t st;
-  AxisPlan px, py, pz;     // any-size kernels: nx / 2, ny, nz
+  AxisPlan px, py, pz;     // any-size kernels: nx, ny / 2, nz
   int zS;                  // z-pass tile of the operator (CG loop)
   int zSr = 8;             // z-pass tile of the residual (fixed-size kernels)
   // workspace
@@ -232,7 +231,7 @@ struct mf_ctx {
   size_t ws_need = 0;
   // offsets into the workspace
   size_t oF, oP, ob, oK, ox, or_, op, op2, oAp, oH, ospec, ophase, oscale, oscale32, otable,
-      otable32, otabledw, opart, osc, ores, oxpos, oxk, oyk, ozk, otw64, otw32, otwdw;
+      otable32, otabledw, opart, osc, ores, oxpos, oxk, oxe, oyk, ozk, otw64, otw32, otwdw;
   // load-history state and tables (history.cu)
   size_t ohist, othout, othin, oFprev, oFprev2;
   int predictor = MF_PRED_UNIFORM;  // mf_set_predictor
@@ -295,7 +294,7 @@ size_t tw_offset(const mf_ctx* c, bool f32, bool dw, size_t* esz) {
 
 XYArgs xy_args(const mf_ctx* c, bool f32, bool dw = false) {
   XYArgs a{};
-  a.v2 = c->v2xy;
+  a.v2 = c->v2;
   a.split = c->xy_split;
   a.skip = nullptr;
   a.fin = 0;
@@ -309,7 +308,7 @@ XYArgs xy_args(const mf_ctx* c, bool f32, bool dw = false) {
   a.flags = &c->at<Scalars>(c->osc)->flags;
   a.nx = c->nx; a.ny = c->ny; a.nz = c->nz; a.N = c->N;
   a.px = c->px; a.py = c->py;
-  a.dny = fast_div(c->ny); a.dh = fast_div(c->nx / 2);
+  a.dhy = fast_div(c->ny / 2); a.dnx = fast_div(c->nx);
   size_t esz;
   const size_t tw = tw_offset(c, f32, dw, &esz);
   a.twx = c->ws + tw;
@@ -321,15 +320,16 @@ XYArgs xy_args(const mf_ctx* c, bool f32, bool dw = false) {
 ZArgs z_args(const mf_ctx* c, bool f32, const uint8_t* mask, double scale, bool dw = false) {
   ZArgs a{};
   memset(&a, 0, sizeof(a));
-  a.v2 = c->v2z;
+  a.v2 = c->v2;
   a.pdl = 1;   // the z-pass waits for its predecessor itself
   a.nx = c->nx; a.ny = c->ny; a.nz = c->nz; a.N = c->N;
   a.pz = c->pz;
-  a.dh = fast_div(c->nx / 2);
+  a.dnx = fast_div(c->nx);
   size_t esz;
   const size_t tw = tw_offset(c, f32, dw, &esz);
   a.twz = c->ws + tw + esz * (c->nx + c->ny);
   a.xk = c->at<int>(c->oxk);
+  a.xe = c->at<int>(c->oxe);
   a.yk = c->at<int>(c->oyk);
   a.zk = c->at<int>(c->ozk);
   a.S = c->zS;
@@ -1295,11 +1295,9 @@ int mf_create(mf_ctx** out, int nx, int ny, int nz, int precision, void* stream)
   c->serial = ++g_ctx_serial;
   memset(&c->keep, 0, sizeof(c->keep));
   c->v2 = mf_v2_supported(nx, ny, nz) ? 1 : 0;
-  c->v2xy = (c->v2 || mf_v2_xy(nx, ny)) ? 1 : 0;
-  c->v2z = mf_v2_z(nx, ny, nz) ? 1 : 0;
   c->xy_split = big_plane ? 1 : 0;
   c->st = (cudaStream_t)stream;
-  if (!mf_make_plan(nx / 2, nx, &c->px) || !mf_make_plan(ny, ny, &c->py) || !mf_make_plan(nz, nz, &c->pz)) {
+  if (!mf_make_plan(nx, nx, &c->px) || !mf_make_plan(ny / 2, ny, &c->py) || !mf_make_plan(nz, nz, &c->pz)) {
     delete c;
     return MF_INVALID_ARG;
   }
@@ -1340,6 +1338,7 @@ int mf_create(mf_ctx** out, int nx, int ny, int nz, int precision, void* stream)
   c->ores = take(9 * sizeof(double));
   c->oxpos = take(nx * sizeof(int));
   c->oxk = take(nx * sizeof(int));
+  c->oxe = take(nx * sizeof(int));
   c->oyk = take(ny * sizeof(int));
   c->ozk = take(nz * sizeof(int));
   c->otw64 = take((nx + ny + nz) * sizeof(double2));
@@ -1360,14 +1359,17 @@ int mf_bind_workspace(mf_ctx* c, void* dev, size_t bytes) {
   free_cg_graph(c);
   // host-built tables: digit-reversal maps and twiddles
   const int nx = c->nx, ny = c->ny, nz = c->nz;
-  std::vector<int> xpos(nx, 0), xk(nx, 0), yk(ny, 0), zk(nz, 0);
-  // half-length rows: slot of kx < nx/2; rows hold ky, planes kz in
-  // digit-reversed order of the kernels that serve the axis
-  const int h = nx / 2;
-  for (int k = 0; k < h; ++k) xpos[k] = c->v2xy ? fft2::dif_pos(h, k) : mf_plan_pos(c->px, k);
-  for (int k = 0; k < h; ++k) xk[xpos[k]] = k;
-  for (int k = 0; k < ny; ++k) yk[c->v2xy ? fft2::dif_pos(ny, k) : mf_plan_pos(c->py, k)] = k;
-  for (int k = 0; k < nz; ++k) zk[c->v2z ? fft2::dif_pos(nz, k) : mf_plan_pos(c->pz, k)] = k;
+  std::vector<int> xpos(nx, 0), xk(nx, 0), xe(nx, 0), yk(ny, 0), zk(nz, 0);
+  if (c->v2) {
+    // half-length rows: slot of kx < nx/2; rows hold ky in digit-reversed order
+    const int h = nx / 2;
+    for (int k = 0; k < h; ++k) xpos[k] = fft2::dif_pos(h, k);
+    for (int k = 0; k < h; ++k) xk[xpos[k]] = k;
+    for (int k = 0; k < ny; ++k) yk[fft2::dif_pos(ny, k)] = k;
+    for (int k = 0; k < nz; ++k) zk[fft2::dif_pos(nz, k)] = k;
+  } else {
+    mf_any_size_maps(c->px, c->py, c->pz, xpos.data(), xk.data(), xe.data(), yk.data(), zk.data());
+  }
   std::vector<double2> tw64(nx + ny + nz);
   std::vector<float2> tw32(nx + ny + nz);
   std::vector<dwc> twdw(nx + ny + nz);
@@ -1388,6 +1390,7 @@ int mf_bind_workspace(mf_ctx* c, void* dev, size_t bytes) {
   };
   put(c->oxpos, xpos.data(), nx * sizeof(int));
   put(c->oxk, xk.data(), nx * sizeof(int));
+  put(c->oxe, xe.data(), nx * sizeof(int));
   put(c->oyk, yk.data(), ny * sizeof(int));
   put(c->ozk, zk.data(), nz * sizeof(int));
   put(c->otw64, tw64.data(), tw64.size() * sizeof(double2));

@@ -45,7 +45,7 @@ extern "C" int mf_residual_noalloc(int nx, int ny, int nz, const double* P_dev, 
   for (int c = 0; c < 9; ++c)
     if (mask[c] > 1 || !isfinite(pbar[c])) return MF_INVALID_ARG;
   AxisPlan px, py, pz;
-  if (!mf_make_plan(nx / 2, nx, &px) || !mf_make_plan(ny, ny, &py) || !mf_make_plan(nz, nz, &pz))
+  if (!mf_make_plan(nx, nx, &px) || !mf_make_plan(ny / 2, ny, &py) || !mf_make_plan(nz, nz, &pz))
     return MF_INVALID_ARG;
   cudaStream_t st = (cudaStream_t)stream;
 
@@ -68,12 +68,8 @@ extern "C" int mf_residual_noalloc(int nx, int ny, int nz, const double* P_dev, 
   double* mean = (double*)(base + kSpecBytes + kTableBytes + kPartialBytes);
 
   // index maps and twiddles, rewritten every call (sizes may differ)
-  const int h = nx / 2;
-  std::vector<int> xpos(h), xk(h), yk(ny), zk(nz);
-  for (int k = 0; k < h; ++k) xpos[k] = mf_plan_pos(px, k);
-  for (int k = 0; k < h; ++k) xk[xpos[k]] = k;
-  for (int k = 0; k < ny; ++k) yk[mf_plan_pos(py, k)] = k;
-  for (int k = 0; k < nz; ++k) zk[mf_plan_pos(pz, k)] = k;
+  std::vector<int> xpos(nx), xk(nx), xe(nx), yk(ny / 2), zk(nz);
+  mf_any_size_maps(px, py, pz, xpos.data(), xk.data(), xe.data(), yk.data(), zk.data());
   std::vector<double2> tw(nx + ny + nz);
   int o = 0;
   for (int n : {nx, ny, nz}) {
@@ -86,14 +82,16 @@ extern "C" int mf_residual_noalloc(int nx, int ny, int nz, const double* P_dev, 
   size_t off = 0;
   auto place = [&](size_t bytes) { size_t r = off; off += (bytes + 255) & ~(size_t)255; return r; };
   const size_t o_tw = place(tw.size() * sizeof(double2));
-  const size_t o_xpos = place(h * sizeof(int)), o_xk = place(h * sizeof(int)),
-               o_yk = place(ny * sizeof(int)), o_zk = place(nz * sizeof(int));
+  const size_t o_xpos = place(nx * sizeof(int)), o_xk = place(nx * sizeof(int)),
+               o_xe = place(nx * sizeof(int)), o_yk = place((ny / 2) * sizeof(int)),
+               o_zk = place(nz * sizeof(int));
   if (off > kTableBytes) return MF_TOO_LARGE;
   cudaError_t e = cudaMemcpyAsync(tab + o_tw, tw.data(), tw.size() * sizeof(double2),
                                   cudaMemcpyHostToDevice, st);
-  if (e == cudaSuccess) e = cudaMemcpyAsync(tab + o_xpos, xpos.data(), h * sizeof(int), cudaMemcpyHostToDevice, st);
-  if (e == cudaSuccess) e = cudaMemcpyAsync(tab + o_xk, xk.data(), h * sizeof(int), cudaMemcpyHostToDevice, st);
-  if (e == cudaSuccess) e = cudaMemcpyAsync(tab + o_yk, yk.data(), ny * sizeof(int), cudaMemcpyHostToDevice, st);
+  if (e == cudaSuccess) e = cudaMemcpyAsync(tab + o_xpos, xpos.data(), nx * sizeof(int), cudaMemcpyHostToDevice, st);
+  if (e == cudaSuccess) e = cudaMemcpyAsync(tab + o_xk, xk.data(), nx * sizeof(int), cudaMemcpyHostToDevice, st);
+  if (e == cudaSuccess) e = cudaMemcpyAsync(tab + o_xe, xe.data(), nx * sizeof(int), cudaMemcpyHostToDevice, st);
+  if (e == cudaSuccess) e = cudaMemcpyAsync(tab + o_yk, yk.data(), (ny / 2) * sizeof(int), cudaMemcpyHostToDevice, st);
   if (e == cudaSuccess) e = cudaMemcpyAsync(tab + o_zk, zk.data(), nz * sizeof(int), cudaMemcpyHostToDevice, st);
   // nothing in the pipeline reads scratch before writing it; the mean slot is
   // cleared so that a failed launch cannot hand back the previous call's mean
@@ -109,7 +107,7 @@ extern "C" int mf_residual_noalloc(int nx, int ny, int nz, const double* P_dev, 
   xa.pdl = 0;
   xa.nx = nx; xa.ny = ny; xa.nz = nz; xa.N = N;
   xa.px = px; xa.py = py;
-  xa.dny = fast_div(ny); xa.dh = fast_div(h);
+  xa.dhy = fast_div(ny / 2); xa.dnx = fast_div(nx);
   xa.twx = tab + o_tw;
   xa.twy = tab + o_tw + sizeof(double2) * nx;
   xa.xpos = (const int*)(tab + o_xpos);
@@ -117,9 +115,10 @@ extern "C" int mf_residual_noalloc(int nx, int ny, int nz, const double* P_dev, 
   memset(&za, 0, sizeof(za));
   za.nx = nx; za.ny = ny; za.nz = nz; za.N = N;
   za.pz = pz;
-  za.dh = fast_div(h);
+  za.dnx = fast_div(nx);
   za.twz = tab + o_tw + sizeof(double2) * (nx + ny);
   za.xk = (const int*)(tab + o_xk);
+  za.xe = (const int*)(tab + o_xe);
   za.yk = (const int*)(tab + o_yk);
   za.zk = (const int*)(tab + o_zk);
   za.mask = 0;

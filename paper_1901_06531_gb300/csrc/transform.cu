@@ -11,11 +11,10 @@
 //                 control, inverse along z.
 //   x-y inverse : per (z-plane, component): inverse along y, complex-to-real
 //                 along x, optionally the CG residual update.
-// The fixed-size kernels (transform2.cuh) run where they exist for a plane
-// or a z length, the any-size ones (transformg.cuh) elsewhere; all share the
-// spectrum layout (launch.h).  The x-Nyquist coefficient is never stored
-// because G-hat-star is zero there.  The 1/N of the forward transform is
-// applied once, in the z-pass.
+// The fixed-size kernels (transform2.cuh) run on the grids they exist for,
+// the any-size ones (transformg.cuh) on the others.  The x-Nyquist coefficient
+// is never stored because G-hat-star is zero there.  The 1/N of the forward
+// transform is applied once, in the z-pass.
 #include "common.cuh"
 #include "dw.cuh"
 
@@ -116,17 +115,9 @@ cudaError_t mf_launch_project_part(int which, bool f32, const void* t, void* spe
   return xyi(f32, 3, spec, r, partials, xa, sc, st);
 }
 
-bool mf_v2_z(int nx, int ny, int nz) {
-  const bool ok = nz == 16 || nz == 32 || nz == 48 || nz == 64 || nz == 96 || nz == 128 || nz == 256;
-  return ok && (ny * (nx / 2)) % 8 == 0;   // whole tiles of eight columns
-}
-
-bool mf_v2_xy(int nx, int ny) {
-  return nx == ny && (nx == 16 || nx == 32 || nx == 48 || nx == 64 || nx == 96 || nx == 128);
-}
-
 bool mf_v2_supported(int nx, int ny, int nz) {
-  return (mf_v2_xy(nx, ny) || (nx == 256 && ny == 256)) && mf_v2_z(nx, ny, nz);
+  auto ok = [](int n) { return n == 16 || n == 32 || n == 48 || n == 64 || n == 96 || n == 128 || n == 256; };
+  return nx == ny && ok(nx) && ok(nz);
 }
 
 bool mf_split_supported(int nx) { return nx == 32 || nx == 256; }

@@ -1,8 +1,7 @@
 """The any-size transform kernels against the oracle at sizes where they can
-go wrong: every radix as a first, middle and last stage, one to three stages
-per axis, odd half lengths and odd nz, partial z-pass tiles, planes near the
-shared-memory limit, and grids that combine any-size kernels on one axis with
-fixed-size kernels on the others.  FP64 operator and residual to 1e-12
+go wrong: every pair of stage radices, one to three passes per axis, odd half
+lengths and odd nz, partial z-pass tiles, planes near the shared-memory limit.
+FP64 operator and residual to 1e-12
 relative (one application, no iteration), the FP32 operator within its
 element-wise bound, both as in the operator tests."""
 import numpy as np
@@ -15,23 +14,23 @@ from gpu_util import fp32_operator_error, lib, neohooke_two_phase, rel
 
 pytestmark = pytest.mark.gpu
 
-# (nx, ny, nz)
+# (nx, ny, nz), with the passes (stage radices) of nx, ny / 2 and nz
 SHAPES = [
-    (4, 6, 2),        # the shortest lengths: one stage, radix 2
-    (6, 4, 3),        # odd half length
-    (18, 12, 27),     # 9 | 12 | 9 x 3
-    (24, 18, 16),     # 12 | 9 x 2 with a fixed-size z-pass
-    (36, 54, 6),      # 9 x 2 | 9 x 6
-    (54, 8, 81),      # 27 = 9 x 3 (odd) | 8 | 9 x 9
-    (72, 24, 12),     # 6 x 6 | 6 x 4
-    (162, 4, 9),      # 81 = 9 x 9 (odd)
-    (4, 162, 4),      # 9 x 9 x 2: three stages along y
-    (8, 16, 243),     # 9 x 9 x 3: three stages along z
-    (16, 16, 54),     # fixed-size x-y passes, any-size z-pass
-    (64, 32, 4),      # 8 x 4 | 8 x 4, not square
-    (256, 6, 4),      # 16 x 8
+    (4, 6, 2),        # 4 | 3 | 2: one stage each
+    (6, 4, 3),        # 2x3 | 2 | 3
+    (18, 12, 27),     # 2x3, 3 | 2x3 | 3x3, 3
+    (24, 18, 16),     # 4x2, 3 | 3x3 | 4x4
+    (36, 54, 6),      # 4, 3x3 | 3x3, 3 | 2x3
+    (54, 8, 81),      # 2x3, 3x3 | 4 | 3x3, 3x3
+    (72, 24, 12),     # 4x2, 3x3 | 4x3 | 4x3
+    (162, 4, 9),      # 2x3, 3x3, 3 (three passes along x) | 2 | 3x3
+    (4, 162, 4),      # odd ny / 2 = 81
+    (8, 16, 243),     # 4x2 | 4x2 | 3x3, 3x3, 3
+    (16, 16, 54),     # 4x4 | 4x2 | 2x3, 3x3
+    (64, 32, 4),      # 4, 4x4 | 4x4 | 4
+    (256, 6, 4),      # 4x4, 4x4 | 3 | 4
     (128, 192, 2),    # the largest plane shared memory takes
-    (96, 144, 2),     # 8 x 6 | 12 x 12
+    (96, 144, 2),     # 4x4, 2x3 | 4x2, 3x3 | 2
 ]
 MASK = np.array([0, 0, 0, 1, 1, 0, 1, 1, 1], np.uint8)
 
@@ -71,7 +70,7 @@ def test_operator_and_residual(shape):
 
 @pytest.mark.parametrize("shape", [(18, 12, 27), (6, 4, 3), (24, 18, 16)])
 def test_caller_fields_need_only_their_own_alignment(shape):
-    """Fields of a caller that start between two complex samples: the
+    """Fields of a caller that start 8 bytes off a 16-byte boundary: the
     residual without a context reads and writes them there, with the bits of
     the aligned call."""
     import torch

@@ -13,6 +13,7 @@
 #include "dw.cuh"
 #include "launch.h"
 #include "predict.cuh"
+#include "reduce.cuh"
 
 namespace {
 
@@ -176,25 +177,6 @@ __device__ __forceinline__ bool neohooke_f32(const float (&h)[9], float mu, floa
   return true;
 }
 
-template <int NC>
-__device__ __forceinline__ void block_sum_dw(double (&v)[NC], double* out) {
-  __shared__ double red[NC][32];
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-#pragma unroll
-  for (int c = 0; c < NC; ++c) {
-    double s = v[c];
-    for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
-    if (lane == 0) red[c][warp] = s;
-  }
-  __syncthreads();
-  if (threadIdx.x < NC) {
-    double s = 0.0;
-    for (int w = 0; w < (int)(blockDim.x >> 5); ++w) s += red[threadIdx.x][w];
-    out[threadIdx.x] = s;
-  }
-  __syncthreads();
-}
-
 // Columns of the block partials: F 0-8, P 9-17, and with MOM T = sum P F^T
 // 18-26, S = sum F F^T 27-35 (FP32 products of the high parts: only used to
 // detect null rotations).  P32: P evaluated in FP32 from H and written, in
@@ -313,7 +295,7 @@ __global__ void __launch_bounds__(kThreads, 2) k_constitutive_dw(double* __restr
 #pragma unroll
     for (int c = 0; c < 18; ++c) a[18 + c] = (double)mom[c];
   }
-  block_sum_dw<NC>(a, tot);
+  block_sum<NC>(a, tot);
   if (threadIdx.x < NC) partials[blockIdx.x * NC + threadIdx.x] = tot[threadIdx.x];
 }
 

@@ -13,6 +13,7 @@
 #include "dw.cuh"
 #include "launch.h"
 #include "predict.cuh"
+#include "reduce.cuh"
 
 namespace {
 
@@ -764,7 +765,6 @@ __global__ void __launch_bounds__(kThreads) k_defl_reduce_h(const T* __restrict_
                                                             long long N, const HistState* hs,
                                                             double* __restrict__ partials) {
   if (hs->defl.m == 0) return;
-  __shared__ double red[9][kThreads / 32];
   double acc[9];
 #pragma unroll
   for (int c = 0; c < 9; ++c) acc[c] = 0.0;
@@ -779,18 +779,9 @@ __global__ void __launch_bounds__(kThreads) k_defl_reduce_h(const T* __restrict_
       for (int j = 0; j < 3; ++j)
         acc[3 * i + j] += q[3 * i] * f[3 * j] + q[3 * i + 1] * f[3 * j + 1] + q[3 * i + 2] * f[3 * j + 2];
   }
-#pragma unroll
-  for (int c = 0; c < 9; ++c) {
-    double s = acc[c];
-    for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
-    if ((threadIdx.x & 31) == 0) red[c][threadIdx.x >> 5] = s;
-  }
-  __syncthreads();
-  if (threadIdx.x < 9) {
-    double s = 0.0;
-    for (int w = 0; w < kThreads / 32; ++w) s += red[threadIdx.x][w];
-    partials[blockIdx.x * 9 + threadIdx.x] = s;
-  }
+  __shared__ double tot[9];
+  block_sum<9>(acc, tot);
+  if (threadIdx.x < 9) partials[blockIdx.x * 9 + threadIdx.x] = tot[threadIdx.x];
 }
 
 // What = sum_k (n_k . y) W_k (zero when no rotation is null).
@@ -848,6 +839,28 @@ __global__ void k_defl_apply_h(T* __restrict__ y, const double* __restrict__ F, 
   }
 }
 
+// Block partials of a Newton update: columns 0-8 the sums of the correction,
+// column 9 the block max of abs(dF_v)^2 (a thread's own max in the type of
+// its correction).
+template <typename T>
+__device__ __forceinline__ void store_update_partials(double (&acc)[9], T mx, double* __restrict__ partials) {
+  __shared__ double tot[9];
+  __shared__ T redm[kThreads / 32];
+  for (int o = 16; o > 0; o >>= 1) {
+    const T other = __shfl_xor_sync(0xffffffffu, mx, o);
+    mx = sizeof(T) == 4 ? (T)fmaxf((float)mx, (float)other) : (T)fmax((double)mx, (double)other);
+  }
+  if ((threadIdx.x & 31) == 0) redm[threadIdx.x >> 5] = mx;
+  block_sum<9>(acc, tot);
+  if (threadIdx.x < 9) {
+    partials[blockIdx.x * 10 + threadIdx.x] = tot[threadIdx.x];
+  } else if (threadIdx.x == 9) {
+    double m = 0.0;
+    for (int w = 0; w < kThreads / 32; ++w) m = fmax(m, (double)redm[w]);
+    partials[blockIdx.x * 10 + 9] = m;
+  }
+}
+
 // F += x (minus What F when a rotation is null).  Partials: columns 0-8 the
 // sums of the applied correction, column 9 the block max of abs(dF_v)^2.
 // An FP32 correction without deflation is widened exactly and summed with
@@ -856,7 +869,6 @@ template <typename T>
 __global__ void __launch_bounds__(kThreads) k_newton_update_h(double* __restrict__ F, const T* __restrict__ x,
                                                               long long N, double* __restrict__ partials,
                                                               const HistState* hs, const Scalars* sc) {
-  __shared__ double red[11][kThreads / 32];
   const bool defl = hs->defl.m > 0;
   if (sizeof(T) == 4 && !defl) return;   // k_newton_update_f32_h
   double acc[9];
@@ -909,25 +921,7 @@ __global__ void __launch_bounds__(kThreads) k_newton_update_h(double* __restrict
 #pragma unroll
     for (int c = 0; c < 9; ++c) acc[c] = (double)xs[c] + (double)xc[c];
   }
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-#pragma unroll
-  for (int c = 0; c < 9; ++c) {
-    double s = acc[c];
-    for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
-    if (lane == 0) red[c][warp] = s;
-  }
-  for (int o = 16; o > 0; o >>= 1) mx = fmax(mx, __shfl_xor_sync(0xffffffffu, mx, o));
-  if (lane == 0) red[9][warp] = mx;
-  __syncthreads();
-  if (threadIdx.x < 9) {
-    double s = 0.0;
-    for (int w = 0; w < kThreads / 32; ++w) s += red[threadIdx.x][w];
-    partials[blockIdx.x * 10 + threadIdx.x] = s;
-  } else if (threadIdx.x == 9) {
-    double m = 0.0;
-    for (int w = 0; w < kThreads / 32; ++w) m = fmax(m, red[9][w]);
-    partials[blockIdx.x * 10 + 9] = m;
-  }
+  store_update_partials(acc, mx, partials);
 }
 
 // The common case of k_newton_update_h on its own: an FP32 correction
@@ -947,7 +941,6 @@ __global__ void __launch_bounds__(kThreads, 3) k_newton_update_f32_h(double* __r
   const int its = p0 ? sc->its : -1;
   const float* __restrict__ p = (its > 0) ? ((its & 1) ? p1 : p0) : nullptr;
   const float a = p ? (float)sc->alpha : 0.f;
-  __shared__ double red[11][kThreads / 32];
   float xs[9], xc[9];
 #pragma unroll
   for (int c = 0; c < 9; ++c) { xs[c] = 0.f; xc[c] = 0.f; }
@@ -980,26 +973,10 @@ __global__ void __launch_bounds__(kThreads, 3) k_newton_update_f32_h(double* __r
     }
     mx = fmaxf(mx, n2);
   }
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  double acc[9];
 #pragma unroll
-  for (int c = 0; c < 9; ++c) {
-    double sv = (double)xs[c] + (double)xc[c];
-    for (int o = 16; o > 0; o >>= 1) sv += __shfl_xor_sync(0xffffffffu, sv, o);
-    if (lane == 0) red[c][warp] = sv;
-  }
-  double m = (double)mx;
-  for (int o = 16; o > 0; o >>= 1) m = fmax(m, __shfl_xor_sync(0xffffffffu, m, o));
-  if (lane == 0) red[9][warp] = m;
-  __syncthreads();
-  if (threadIdx.x < 9) {
-    double sv = 0.0;
-    for (int w = 0; w < kThreads / 32; ++w) sv += red[threadIdx.x][w];
-    partials[blockIdx.x * 10 + threadIdx.x] = sv;
-  } else if (threadIdx.x == 9) {
-    double mm = 0.0;
-    for (int w = 0; w < kThreads / 32; ++w) mm = fmax(mm, red[9][w]);
-    partials[blockIdx.x * 10 + 9] = mm;
-  }
+  for (int c = 0; c < 9; ++c) acc[c] = (double)xs[c] + (double)xc[c];
+  store_update_partials(acc, mx, partials);
 }
 
 // The solve's last lagging update x += alpha p (k_axpy_last) for an FP32

@@ -8,32 +8,11 @@
 
 #include "dw.cuh"
 #include "launch.h"
+#include "reduce.cuh"
 
 namespace {
 
 constexpr int kRedThreads = 256;
-
-// Sum NC columns over the block; thread 0..NC-1 of warp 0 end up holding the
-// totals in out[col] (a shared array).
-template <int NC>
-__device__ __forceinline__ void block_sum(double (&v)[NC], double* out) {
-  __shared__ double red[NC][32];
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-#pragma unroll
-  for (int c = 0; c < NC; ++c) {
-    double s = v[c];
-    for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
-    if (lane == 0) red[c][warp] = s;
-  }
-  __syncthreads();
-  if (threadIdx.x < NC) {
-    double s = 0.0;
-    const int nw = blockDim.x >> 5;
-    for (int w = 0; w < nw; ++w) s += red[threadIdx.x][w];
-    out[threadIdx.x] = s;
-  }
-  __syncthreads();
-}
 
 // Deterministic column sums of partials[nblk][ncol] by one block.
 __device__ __forceinline__ double column_sum(const double* partials, int nblk, int ncol, int col,

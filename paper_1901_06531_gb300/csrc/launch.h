@@ -201,6 +201,8 @@ cudaError_t mf_launch_constitutive_dw(const double* F, double* P, float* H, bool
                                       const void* table_dw, long long N, double* partials, int nblk,
                                       Scalars* sc, cudaStream_t st, float* Pf = nullptr,
                                       const float* table32 = nullptr, const PredArgs* pred = nullptr);
+// F = I everywhere (N even)
+cudaError_t mf_launch_identity(double* F, long long N, cudaStream_t st);
 cudaError_t mf_launch_mean_F(const double* F, long long N, double* partials, int nblk, Scalars* sc,
                              cudaStream_t st);
 cudaError_t mf_launch_predictor(double* F, long long N, const uint8_t* mask9, const double* target9,

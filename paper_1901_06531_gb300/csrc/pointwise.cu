@@ -249,6 +249,19 @@ __global__ void __launch_bounds__(kRedThreads) k_mean_F(const double* __restrict
   if (threadIdx.x < 9) partials[blockIdx.x * 9 + threadIdx.x] = tot[threadIdx.x];
 }
 
+// F = I, two values per store (N is even and the field 256-byte aligned).
+__global__ void __launch_bounds__(kRedThreads) k_identity(double2* __restrict__ F, long long N) {
+  const long long h = N / 2;
+  for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < h;
+       i += (long long)gridDim.x * blockDim.x) {
+#pragma unroll
+    for (int c = 0; c < 9; ++c) {
+      const double d = (c % 4 == 0) ? 1.0 : 0.0;
+      F[c * h + i] = make_double2(d, d);
+    }
+  }
+}
+
 struct Load9 {
   double target[9];
   unsigned char mask[9];
@@ -515,6 +528,12 @@ cudaError_t mf_launch_constitutive(const double* F, double* P, void* K45, bool k
     k_fin_means<<<ncol, kRedThreads, 0, st>>>(partials, nblk, ncol, N, sc);
   }
   g_mf_launches += 2;
+  return cudaGetLastError();
+}
+
+cudaError_t mf_launch_identity(double* F, long long N, cudaStream_t st) {
+  k_identity<<<stride_grid(N / 2, kRedThreads), kRedThreads, 0, st>>>(reinterpret_cast<double2*>(F), N);
+  g_mf_launches += 1;
   return cudaGetLastError();
 }
 

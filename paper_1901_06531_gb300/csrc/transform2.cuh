@@ -735,7 +735,7 @@ __global__ void __launch_bounds__(z_threads(S_), z_min_blocks<T>(S_, MODE)) k_zp
       v2 = cmake(q.x * xi2, q.y * xi2);
     }
   };
-  if constexpr (sizeof(C) == 8) {
+  if constexpr (sizeof(C) == 8 && NST > 1) {
     // FP32: last forward stage, G-hat-star and first inverse stage in
     // registers (three components of RL positions of one column per thread)
     constexpr int NB = NZ / RL;
@@ -747,7 +747,7 @@ __global__ void __launch_bounds__(z_threads(S_), z_min_blocks<T>(S_, MODE)) k_zp
 #pragma unroll
         for (int r = 0; r < RL; ++r) {
           const int z = blk * RL + r;
-          v[cl][r] = (NST > 1) ? buf[MF_AT(cl * CP + z * ZS + s, 3 * CP)] : gsp[gidx(cl * S + s, z)];
+          v[cl][r] = buf[MF_AT(cl * CP + z * ZS + s, 3 * CP)];
         }
 #pragma unroll
       for (int cl = 0; cl < 3; ++cl) fft2::Dft<RL, false, C>::run(v[cl]);
@@ -760,14 +760,15 @@ __global__ void __launch_bounds__(z_threads(S_), z_min_blocks<T>(S_, MODE)) k_zp
 #pragma unroll
         for (int r = 0; r < RL; ++r) {
           const int z = blk * RL + r;
-          if (NST > 1) buf[MF_AT(cl * CP + z * ZS + s, 3 * CP)] = v[cl][r];
-          else gsp[gidx(cl * S + s, z)] = v[cl][r];
+          buf[MF_AT(cl * CP + z * ZS + s, 3 * CP)] = v[cl][r];
         }
     }
   } else {
     // 16-byte types (FP64, double word): registers are scarcer, so the last
     // forward stage, G-hat-star and the first inverse stage are separate
-    // passes over shared memory
+    // passes over shared memory.  So they are for nz = 16 in FP32, one radix-16
+    // stage: in registers it left eight threads a block with all the work
+    // (three transforms and sixteen G-hat-star evaluations each, 14 us a launch)
     if constexpr (NST == 1) {
       for (int idx = threadIdx.x; idx < 3 * NZ * S; idx += kZThreads) {
         const int s2 = idx % S, cz = idx / S, cl = cz / NZ, z = cz - cl * NZ;

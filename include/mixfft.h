@@ -349,7 +349,7 @@ int mf_selftest_wait_timeout(int max_polls);
  * plane, 1 persistent, 2 cluster); xy_ms_out: host 2 floats or NULL, mean ms
  * of the forward pass per plane and persistent (-1 when not timed; all five
  * timings through mf_xy_schedule).
- * Contexts served by the generic kernels keep their fixed tile. */
+ * Contexts served by the any-size kernels keep their tile (ms_out -1). */
 int mf_autotune(mf_ctx* ctx, int32_t* zs_out, float* ms_out, int32_t* xy_out, float* xy_ms_out);
 
 /* Adjoint sensitivity of the homogenized response at the current F, which

@@ -220,7 +220,8 @@ struct mf_ctx {
   int nx, ny, nz;
   long long N;
   int prec;
-  int v2 = 0;              // fixed-size transform kernels and their table layout
+  int v2_ok = 0;           // the fixed-size transform kernels exist for the grid
+  int v2 = 0;              // they (and their table layout) are used
   int xy_split = 0;        // with v2: separate row and column kernels for the x-y transform
   cudaStream_t st;
   AxisPlan px, py, pz;     // any-size kernels: nx, ny / 2, nz
@@ -277,6 +278,17 @@ struct mf_ctx {
 };
 
 namespace {
+
+// Whether a context whose grid has fixed-size kernels uses them.  FP32-inner
+// contexts do.  Plain FP64 is bound by the FP64 pipe, or on small cells by how
+// many threads share its chains: per CG iteration the any-size kernels take
+// 44, 74, 190 and 1503 us against 58, 95, 256 and 1562 us on 16^3, 32^3, 48^3
+// and 96^3, but 474 against 430 us on 64^3 (8 x 8 stages), so planes of 64^2,
+// 128^2 and 256^2 stay with the fixed-size ones.
+int use_fixed_size(const mf_ctx* c) {
+  if (!c->v2_ok) return 0;
+  return (c->f32() || c->nx == 64 || c->nx == 128 || c->nx == 256) ? 1 : 0;
+}
 
 char g_last_cuda_error[256] = "";
 
@@ -1245,6 +1257,50 @@ int solve_cell(mf_ctx* c, int nsteps, const uint8_t* mask, const double* target,
   return MF_OK;
 }
 
+// Host-built tables of a context: digit-reversal maps and twiddles.
+int upload_tables(mf_ctx* c) {
+  const int nx = c->nx, ny = c->ny, nz = c->nz;
+  std::vector<int> xpos(nx, 0), xk(nx, 0), xe(nx, 0), yk(ny, 0), zk(nz, 0);
+  if (c->v2) {
+    // half-length rows: slot of kx < nx/2; rows hold ky in digit-reversed order
+    const int h = nx / 2;
+    for (int k = 0; k < h; ++k) xpos[k] = fft2::dif_pos(h, k);
+    for (int k = 0; k < h; ++k) xk[xpos[k]] = k;
+    for (int k = 0; k < ny; ++k) yk[fft2::dif_pos(ny, k)] = k;
+    for (int k = 0; k < nz; ++k) zk[fft2::dif_pos(nz, k)] = k;
+  } else {
+    mf_any_size_maps(c->px, c->py, c->pz, xpos.data(), xk.data(), xe.data(), yk.data(), zk.data());
+  }
+  std::vector<double2> tw64(nx + ny + nz);
+  std::vector<float2> tw32(nx + ny + nz);
+  std::vector<dwc> twdw(nx + ny + nz);
+  int o = 0;
+  for (int n : {nx, ny, nz}) {
+    for (int t = 0; t < n; ++t) {
+      const double ang = -2.0 * M_PI * (double)t / (double)n;
+      tw64[o + t] = make_double2(cos(ang), sin(ang));
+      tw32[o + t] = make_float2((float)tw64[o + t].x, (float)tw64[o + t].y);
+      twdw[o + t].x = dw(tw64[o + t].x);
+      twdw[o + t].y = dw(tw64[o + t].y);
+    }
+    o += n;
+  }
+  cudaError_t e = cudaSuccess;
+  auto put = [&](size_t off, const void* src, size_t bytes) {
+    if (e == cudaSuccess) e = cudaMemcpyAsync(c->ws + off, src, bytes, cudaMemcpyHostToDevice, c->st);
+  };
+  put(c->oxpos, xpos.data(), nx * sizeof(int));
+  put(c->oxk, xk.data(), nx * sizeof(int));
+  put(c->oxe, xe.data(), nx * sizeof(int));
+  put(c->oyk, yk.data(), ny * sizeof(int));
+  put(c->ozk, zk.data(), nz * sizeof(int));
+  put(c->otw64, tw64.data(), tw64.size() * sizeof(double2));
+  put(c->otw32, tw32.data(), tw32.size() * sizeof(float2));
+  put(c->otwdw, twdw.data(), twdw.size() * sizeof(dwc));
+  if (e == cudaSuccess) e = cudaStreamSynchronize(c->st);   // host vectors go out of scope
+  return cuda_status(e);
+}
+
 int check_solve_args(const mf_ctx* c, int nsteps, const uint8_t* mask, const double* target, double tol_newton,
                      double tol_cg, double cg_rel, int max_newton, int max_cg) {
   if (!c || nsteps < 0 || (nsteps > 0 && (!mask || !target)) || !(tol_newton > 0) || !(tol_cg > 0) ||
@@ -1294,10 +1350,17 @@ int mf_create(mf_ctx** out, int nx, int ny, int nz, int precision, void* stream)
   c->prec = precision;
   c->serial = ++g_ctx_serial;
   memset(&c->keep, 0, sizeof(c->keep));
-  c->v2 = mf_v2_supported(nx, ny, nz) ? 1 : 0;
+  c->v2_ok = mf_v2_supported(nx, ny, nz) ? 1 : 0;
+  c->v2 = use_fixed_size(c);
   c->xy_split = big_plane ? 1 : 0;
   c->st = (cudaStream_t)stream;
-  if (!mf_make_plan(nx, nx, &c->px) || !mf_make_plan(ny / 2, ny, &c->py) || !mf_make_plan(nz, nz, &c->pz)) {
+  // any-size passes: small FP64 cells one stage at a time, which keeps four
+  // times the threads busy with a quarter of the serial FP64 chain each (per
+  // CG iteration: 16^3 63 -> 44 us, 24^3 63 -> 56, 32^3 80 -> 74; at 36^3 the
+  // pairs win, 127 against 139)
+  const bool pairs = !(precision == MF_FP64 && c->N <= 32 * 32 * 32);
+  if (!mf_make_plan(nx, nx, pairs, &c->px) || !mf_make_plan(ny / 2, ny, pairs, &c->py) ||
+      !mf_make_plan(nz, nz, pairs, &c->pz)) {
     delete c;
     return MF_INVALID_ARG;
   }
@@ -1357,48 +1420,9 @@ int mf_bind_workspace(mf_ctx* c, void* dev, size_t bytes) {
   c->model = -1;
   c->have_K = false;
   free_cg_graph(c);
-  // host-built tables: digit-reversal maps and twiddles
-  const int nx = c->nx, ny = c->ny, nz = c->nz;
-  std::vector<int> xpos(nx, 0), xk(nx, 0), xe(nx, 0), yk(ny, 0), zk(nz, 0);
-  if (c->v2) {
-    // half-length rows: slot of kx < nx/2; rows hold ky in digit-reversed order
-    const int h = nx / 2;
-    for (int k = 0; k < h; ++k) xpos[k] = fft2::dif_pos(h, k);
-    for (int k = 0; k < h; ++k) xk[xpos[k]] = k;
-    for (int k = 0; k < ny; ++k) yk[fft2::dif_pos(ny, k)] = k;
-    for (int k = 0; k < nz; ++k) zk[fft2::dif_pos(nz, k)] = k;
-  } else {
-    mf_any_size_maps(c->px, c->py, c->pz, xpos.data(), xk.data(), xe.data(), yk.data(), zk.data());
-  }
-  std::vector<double2> tw64(nx + ny + nz);
-  std::vector<float2> tw32(nx + ny + nz);
-  std::vector<dwc> twdw(nx + ny + nz);
-  int o = 0;
-  for (int n : {nx, ny, nz}) {
-    for (int t = 0; t < n; ++t) {
-      const double ang = -2.0 * M_PI * (double)t / (double)n;
-      tw64[o + t] = make_double2(cos(ang), sin(ang));
-      tw32[o + t] = make_float2((float)tw64[o + t].x, (float)tw64[o + t].y);
-      twdw[o + t].x = dw(tw64[o + t].x);
-      twdw[o + t].y = dw(tw64[o + t].y);
-    }
-    o += n;
-  }
-  cudaError_t e = cudaSuccess;
-  auto put = [&](size_t off, const void* src, size_t bytes) {
-    if (e == cudaSuccess) e = cudaMemcpyAsync(c->ws + off, src, bytes, cudaMemcpyHostToDevice, c->st);
-  };
-  put(c->oxpos, xpos.data(), nx * sizeof(int));
-  put(c->oxk, xk.data(), nx * sizeof(int));
-  put(c->oxe, xe.data(), nx * sizeof(int));
-  put(c->oyk, yk.data(), ny * sizeof(int));
-  put(c->ozk, zk.data(), nz * sizeof(int));
-  put(c->otw64, tw64.data(), tw64.size() * sizeof(double2));
-  put(c->otw32, tw32.data(), tw32.size() * sizeof(float2));
-  put(c->otwdw, twdw.data(), twdw.size() * sizeof(dwc));
-  if (e == cudaSuccess) e = cudaMemsetAsync(c->ws + c->osc, 0, sizeof(Scalars), c->st);
-  if (e == cudaSuccess) e = cudaStreamSynchronize(c->st);   // host vectors go out of scope
-  return cuda_status(e);
+  const cudaError_t e = cudaMemsetAsync(c->ws + c->osc, 0, sizeof(Scalars), c->st);
+  if (e != cudaSuccess) return cuda_status(e);
+  return upload_tables(c);
 }
 
 int mf_set_material(mf_ctx* c, int model, int nphase, const double* params, const double* rot,
@@ -1921,11 +1945,18 @@ int mf_adjoint(mf_ctx* c, const uint8_t* mask, const double* wF, const double* w
 
 int mf_set_xy_split(mf_ctx* c, int split) {
   if (!c || (split != 0 && split != 1)) return MF_INVALID_ARG;
-  if (split && !(c->v2 && mf_split_supported(c->nx))) return MF_INVALID_ARG;
+  if (split && !(c->v2_ok && mf_split_supported(c->nx))) return MF_INVALID_ARG;
   const bool big_plane = (size_t)(c->ny / 2) * c->nx * sizeof(double2) + (size_t)(c->nx + c->ny) * 20 > 200 * 1024;
   if (!split && big_plane) return MF_INVALID_ARG;
   if (c->xy_split != split) free_cg_graph(c);   // the captured loop holds the old kernels
   c->xy_split = split;
+  // the split kernels have the fixed-size kernels' layout
+  const int v2 = split ? 1 : use_fixed_size(c);
+  if (v2 != c->v2) {
+    c->v2 = v2;
+    c->tuned = false;
+    if (c->ws) return upload_tables(c);
+  }
   return MF_OK;
 }
 
@@ -2095,6 +2126,8 @@ int mf_autotune(mf_ctx* c, int32_t* zs_out, float* ms_out, int32_t* xy_out, floa
   const int s = autotune(c, 5);
   if (s) return s;
   if (zs_out) *zs_out = c->zS;
+  if (ms_out && !c->v2)
+    for (int i = 0; i < 3; ++i) ms_out[i] = -1.f;   // nothing to choose
   if (ms_out) {
     std::lock_guard<std::mutex> lk(g_tune_mutex);
     for (const TuneEntry& t : g_tune_cache)

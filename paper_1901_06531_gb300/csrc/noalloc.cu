@@ -45,7 +45,7 @@ extern "C" int mf_residual_noalloc(int nx, int ny, int nz, const double* P_dev, 
   for (int c = 0; c < 9; ++c)
     if (mask[c] > 1 || !isfinite(pbar[c])) return MF_INVALID_ARG;
   AxisPlan px, py, pz;
-  if (!mf_make_plan(nx, nx, &px) || !mf_make_plan(ny / 2, ny, &py) || !mf_make_plan(nz, nz, &pz))
+  if (!mf_make_plan(nx, nx, true, &px) || !mf_make_plan(ny / 2, ny, true, &py) || !mf_make_plan(nz, nz, true, &pz))
     return MF_INVALID_ARG;
   cudaStream_t st = (cudaStream_t)stream;
 

@@ -16,7 +16,7 @@ inline bool mf_smooth_size(int n) {
 // of length ntab (a multiple of n): stages of radix 4, then 2, then 3, two to
 // a pass; of an odd number of stages the first or the last is a pass of its
 // own, whichever leaves the smaller largest pass.
-inline bool mf_make_plan(int n, int ntab, AxisPlan* p) {
+inline bool mf_make_plan(int n, int ntab, bool pairs, AxisPlan* p) {
   p->n = n;
   p->ntab = ntab;
   p->nst = 0;
@@ -40,7 +40,7 @@ inline bool mf_make_plan(int n, int ntab, AxisPlan* p) {
     if (p->npass >= MF_MAX_PASSES) return false;
     AxisPass& g = p->pass[p->npass++];
     g.r1 = p->rad[s];
-    g.r2 = (s >= start && s + 1 < p->nst) ? p->rad[s + 1] : 1;
+    g.r2 = (pairs && s >= start && s + 1 < p->nst) ? p->rad[s + 1] : 1;
     g.tstep1 = ntab / L;
     g.tstep2 = ntab / (L / g.r1);
     s += g.r2 > 1 ? 2 : 1;

@@ -128,8 +128,11 @@ __device__ __forceinline__ void load_tables(C* twx, C* twy, int* posx, const XYA
 }
 
 // Forward x-y transform of one (c, z) plane per block.
+// Registers: 64 a thread in FP32 (two blocks of 512 an SM), 128 in FP64.
+template <typename T> __host__ __device__ constexpr int xy_min_blocks() { return sizeof(T) == 4 ? 2 : 1; }
+
 template <typename T>
-__global__ void __launch_bounds__(512) k_xyf(const T* __restrict__ in, typename CT<T>::t* __restrict__ spec, XYArgs a) {
+__global__ void __launch_bounds__(512, xy_min_blocks<T>()) k_xyf(const T* __restrict__ in, typename CT<T>::t* __restrict__ spec, XYArgs a) {
   typedef typename CT<T>::t C;
   extern __shared__ __align__(16) unsigned char smem_raw[];
   const int nx = a.nx, ny = a.ny, hy = ny / 2, hx = nx / 2, PX = pitch(nx);
@@ -194,7 +197,7 @@ __global__ void __launch_bounds__(512) k_xyf(const T* __restrict__ in, typename 
 // the last block to finish sums the partials and updates beta, r.r and the
 // stop flag.
 template <typename T, int MODE>
-__global__ void __launch_bounds__(512) k_xyi(const typename CT<T>::t* __restrict__ spec, T* __restrict__ out,
+__global__ void __launch_bounds__(512, xy_min_blocks<T>()) k_xyi(const typename CT<T>::t* __restrict__ spec, T* __restrict__ out,
                                              double* __restrict__ partials, XYArgs a, Scalars* sc) {
   typedef typename CT<T>::t C;
   extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -212,6 +215,12 @@ __global__ void __launch_bounds__(512) k_xyi(const typename CT<T>::t* __restrict
   (void)ext;
   T* dst = out + c * a.N + (long long)z * ny * nx;
   const C* src = spec + ((long long)c * a.nz + z) * half;
+  if (MODE == 3) {
+    // the residual plane is read only at the end: start pulling it into L2 now
+    const char* rp = reinterpret_cast<const char*>(dst);
+    for (int i = threadIdx.x * 128; i < ny * nx * (int)sizeof(T); i += blockDim.x * 128)
+      asm volatile("prefetch.global.L2 [%0];" ::"l"(rp + i));
+  }
   __syncthreads();   // tables
   // y: the first inverse pass reads the spectrum
   pass<C, true, true>(a.py, a.py.npass - 1, nx, a.dnx, twy, [&](int q, int e) { return src[MF_AT(e * nx + q, half)]; },
@@ -410,11 +419,43 @@ __global__ void __launch_bounds__(256) k_zp(typename CT<T>::t* __restrict__ spec
 }
 
 // ---------------------------------------------------------------- launchers
-// Threads of an x-y block: about one eight-value butterfly each, so that
-// small planes share an SM.
-inline int xy_threads(const XYArgs& a) {
-  const int t = ((a.ny * (a.nx / 2) / 8 + 31) / 32) * 32;
-  return t < 64 ? 64 : (t > 512 ? 512 : t);
+// Threads of a block of a grid of `blocks`, at most one per butterfly
+// (`work`): of the counts that run the grid in the fewest waves of resident
+// blocks, the largest.  The phases of a block alternate with barriers, so an
+// SM wants several blocks, and a last wave of a few blocks costs a whole one:
+// 72^3 in FP32 (648 planes) takes 160 us per CG iteration with 352 threads
+// (two blocks an SM, 2.1 waves) and 137 us with 192 (five, one wave), 108^3
+// 406 us with 512 and 391 us with 256.
+inline int pick_threads(int regs, size_t smem, int blocks, int work, int most) {
+  work = ((work + 31) / 32) * 32;
+  most = work < 64 ? 64 : (work < most ? work : most);
+  const int r8 = ((regs + 7) / 8) * 8;
+  int best = 64, fewest = 1 << 30;
+  for (int t = 64; t <= most; t += 32) {
+    int res = 65536 / (r8 * t);
+    const int by_smem = (int)(228 * 1024 / (smem + 1024)), by_warps = 2048 / t;
+    if (by_smem < res) res = by_smem;
+    if (by_warps < res) res = by_warps;
+    if (res > 32) res = 32;
+    if (res < 1) continue;
+    const int waves = (blocks + 152 * res - 1) / (152 * res);
+    if (waves <= fewest) { fewest = waves; best = t; }
+  }
+  return best;
+}
+
+template <auto K> int regs_of() {
+  static const int n = [] {
+    cudaFuncAttributes at;
+    return cudaFuncGetAttributes(&at, K) == cudaSuccess ? at.numRegs : 128;
+  }();
+  return n;
+}
+
+// Values of a butterfly: eight in plans of paired stages, else four.
+inline int xy_work(const XYArgs& a) {
+  const bool paired = a.px.npass < a.px.nst || a.py.npass < a.py.nst;
+  return a.ny * (a.nx / 2) / (paired ? 8 : 4);
 }
 
 template <typename T>
@@ -440,7 +481,8 @@ cudaError_t xyf(const void* in, void* spec, const XYArgs& a, cudaStream_t st) {
   const size_t sm = xy_smem<T>(a);
   if (sm > kSmemMax) return cudaErrorInvalidValue;
   ++g_mf_launches;
-  return launch_k(a.pdl != 0, k_xyf<T>, dim3(9 * a.nz), dim3(xy_threads(a)), sm, st, (const T*)in, (C*)spec, a);
+  const int t = pick_threads(regs_of<k_xyf<T>>(), sm, 9 * a.nz, xy_work(a), 512);
+  return launch_k(a.pdl != 0, k_xyf<T>, dim3(9 * a.nz), dim3(t), sm, st, (const T*)in, (C*)spec, a);
 }
 
 template <typename T, int MODE>
@@ -451,8 +493,9 @@ cudaError_t xyi_m(const void* spec, void* out, double* partials, const XYArgs& a
   const size_t sm = xy_smem<T>(a);
   if (sm > kSmemMax) return cudaErrorInvalidValue;
   ++g_mf_launches;
-  return launch_k(a.pdl != 0, k_xyi<T, MODE>, dim3(9 * a.nz), dim3(xy_threads(a)), sm, st, (const C*)spec, (T*)out,
-                  partials, a, const_cast<Scalars*>(sc));
+  const int t = pick_threads(regs_of<k_xyi<T, MODE>>(), sm, 9 * a.nz, xy_work(a), 512);
+  return launch_k(a.pdl != 0, k_xyi<T, MODE>, dim3(9 * a.nz), dim3(t), sm, st, (const C*)spec, (T*)out, partials, a,
+                  const_cast<Scalars*>(sc));
 }
 
 template <typename T>
@@ -470,10 +513,10 @@ cudaError_t zp_s(void* spec, ZArgs a, cudaStream_t st) {
   if (sm > kSmemMax) return cudaErrorInvalidValue;
   const int ncol = a.ny * (a.nx / 2);
   a.dseq = fast_div(3 * S);
-  int t = ((3 * S * a.nz / 8 + 31) / 32) * 32;   // about one eight-value butterfly per thread
-  t = t < 64 ? 64 : (t > 256 ? 256 : t);
+  const int blocks = 3 * ((ncol + S - 1) / S);
+  const int t = pick_threads(regs_of<k_zp<T, MODE, S>>(), sm, blocks, 3 * S * a.nz / (a.pz.npass < a.pz.nst ? 8 : 4), 256);
   ++g_mf_launches;
-  return launch_k(a.pdl != 0, k_zp<T, MODE, S>, dim3(3 * ((ncol + S - 1) / S)), dim3(t), sm, st, (C*)spec, a);
+  return launch_k(a.pdl != 0, k_zp<T, MODE, S>, dim3(blocks), dim3(t), sm, st, (C*)spec, a);
 }
 
 // Tile of 8 columns; of 4 when 8 would leave SMs without a block.

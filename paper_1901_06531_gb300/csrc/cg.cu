@@ -157,8 +157,10 @@ __device__ __forceinline__ void neohooke_apply(const float (&h)[9], float mu, fl
 // CG true: p = r + beta p', x += alpha' p' first (p' = pin); false: p = pin.
 // FIN (with CG): the last block to finish sums the partials of p.t and sets
 // alpha (no separate finishing launch).
+// Registers: TAN 0 two blocks of 256 an SM (its 45 tangent entries in flight),
+// the others four, five without the CG vectors.
 template <typename T, int TAN, bool CG, bool FIN>
-__global__ void __launch_bounds__(kThreads) k_tangent(const T* __restrict__ pin, const T* __restrict__ r,
+__global__ void __launch_bounds__(kThreads, TAN == 0 ? 2 : (CG ? 4 : 5)) k_tangent(const T* __restrict__ pin, const T* __restrict__ r,
                                                       T* __restrict__ pout, T* __restrict__ x,
                                                       TangentArgs ta, T* __restrict__ t, long long N,
                                                       double* __restrict__ partials, Scalars* sc) {
@@ -168,10 +170,24 @@ __global__ void __launch_bounds__(kThreads) k_tangent(const T* __restrict__ pin,
   pdl_wait();
   bool first = false;   // first CG iteration: p = r, x = 0 (neither previous vector is read)
   if (CG) {
-    if (*(volatile const int*)&sc->stop) return;
-    beta = (T)sc->beta;
-    alpha = (T)sc->alpha;
-    first = sc->its == 0;
+    // the four scalars in one memory latency, read by one thread: the block
+    // scalars share an L2 line, which a read per warp turns into a queue
+    // (64^3, 8192 warps)
+    __shared__ int s_stop, s_its;
+    __shared__ T s_beta, s_alpha;
+    if (threadIdx.x == 0) {
+      const int stop = *(volatile const int*)&sc->stop, its = *(volatile const int*)&sc->its;
+      const double b = *(volatile const double*)&sc->beta, a = *(volatile const double*)&sc->alpha;
+      s_stop = stop;
+      s_its = its;
+      s_beta = (T)b;
+      s_alpha = (T)a;
+    }
+    __syncthreads();
+    if (s_stop) return;
+    beta = s_beta;
+    alpha = s_alpha;
+    first = s_its == 0;
   }
   double acc64 = 0.0;
   Dot32 acc32;
@@ -195,10 +211,15 @@ __global__ void __launch_bounds__(kThreads) k_tangent(const T* __restrict__ pin,
         for (int c = 0; c < 9; ++c) { rv[c] = r[c * N + v]; xv[c] = x[c * N + v]; }
       }
     }
+    T kv[TAN == 0 ? 45 : 1];
     if (TAN != 0) {
 #pragma unroll
       for (int c = 0; c < 9; ++c) h[c] = ta.H[c * N + v];
       ph = ta.phase[v];
+    } else {
+      const T* K = reinterpret_cast<const T*>(ta.K45);
+#pragma unroll
+      for (int t = 0; t < 45; ++t) kv[t] = K[t * N + v];
     }
     T q[9];
 #pragma unroll
@@ -213,14 +234,16 @@ __global__ void __launch_bounds__(kThreads) k_tangent(const T* __restrict__ pin,
     }
     T o[9];
     if (TAN == 0) {
-      const T* K = reinterpret_cast<const T*>(ta.K45);
+      // every entry loaded once, each used for its row and its column
 #pragma unroll
-      for (int a = 0; a < 9; ++a) {
-        T s = (T)0;
+      for (int a = 0; a < 9; ++a) o[a] = kv[sym45(a, a)] * q[a];
 #pragma unroll
-        for (int b = 0; b < 9; ++b) s += K[(long long)sym45(a, b) * N + v] * q[b];
-        o[a] = s;
-      }
+      for (int a = 0; a < 9; ++a)
+#pragma unroll
+        for (int b = a + 1; b < 9; ++b) {
+          o[a] += kv[sym45(a, b)] * q[b];
+          o[b] += kv[sym45(a, b)] * q[a];
+        }
     } else {
       float qf[9], tf[9];
 #pragma unroll

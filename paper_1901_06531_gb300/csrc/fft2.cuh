@@ -202,6 +202,43 @@ __device__ __forceinline__ void stage_io(const C* __restrict__ tw, LD ld, ST st)
   }
 }
 
+// stage_io whose outputs are combined with values of their own places,
+// pre(q, e), all loaded before the butterfly runs: a read-modify-write of
+// global memory then waits for its loads once, not once per output.
+template <typename C, int N, int NTAB, int S, bool INV, int NSEQ, int SQ, int SQSTR, int SSTR,
+          int ESTR, bool SEQFAST, typename LD, typename PRE, typename ST>
+__device__ __forceinline__ void stage_rmw(const C* __restrict__ tw, LD ld, PRE pre, ST st) {
+  constexpr int R = rad(N, S), L = len(N, S), M = L / R, NB = N / R, TSTEP = NTAB / L;
+  for (int t = threadIdx.x; t < NSEQ * NB; t += blockDim.x) {
+    int q, b;
+    if (SEQFAST) { q = t % NSEQ; b = t / NSEQ; } else { b = t % NB; q = t / NB; }
+    const int blk = b / M;
+    const int j0 = b - blk * M;
+    const int base = (q / SQ) * SQSTR + (q % SQ) * SSTR + (blk * L + j0) * ESTR;
+    const int e0 = blk * L + j0;
+    C v[R], w[R];
+#pragma unroll
+    for (int r = 0; r < R; ++r) w[r] = pre(q, e0 + r * M);
+#pragma unroll
+    for (int r = 0; r < R; ++r) v[r] = ld(q, base + r * M * ESTR, e0 + r * M);
+    if (!INV) {
+      Dft<R, false, C>::run(v);
+      if (M > 1) {
+#pragma unroll
+        for (int k = 1; k < R; ++k) v[k] = cmul(v[k], tw[MF_AT(j0 * k * TSTEP, NTAB)]);
+      }
+    } else {
+      if (M > 1) {
+#pragma unroll
+        for (int k = 1; k < R; ++k) v[k] = cmulc(v[k], tw[MF_AT(j0 * k * TSTEP, NTAB)]);
+      }
+      Dft<R, true, C>::run(v);
+    }
+#pragma unroll
+    for (int r = 0; r < R; ++r) st(q, e0 + r * M, v[r], w[r]);
+  }
+}
+
 // Largest shared-memory index a stage over this layout touches, plus one:
 // the extent the debug build checks stage() accesses against.
 template <int N, int NSEQ, int SQ, int SQSTR, int SSTR, int ESTR>

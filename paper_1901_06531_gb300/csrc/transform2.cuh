@@ -46,10 +46,11 @@ constexpr int kXY128Threads = 512;
 template <typename T, int NX> __host__ __device__ constexpr int xy_threads() {
   return sizeof(typename CT<T>::t) == 16 ? 512 : (NX == 128 ? kXY128Threads : 256);
 }
-// resident blocks per SM the register allocation of an FP32 128 x 128 x-y
-// kernel is held to when it runs 512 threads: two (64 registers a thread)
+// resident blocks per SM the register allocation of an FP32 x-y kernel is
+// held to: two of 512 threads (128 x 128 planes, 64 registers a thread),
+// three of 256
 template <typename T, int NX> __host__ __device__ constexpr int xy_min_blocks() {
-  return (sizeof(typename CT<T>::t) == 8 && NX == 128 && kXY128Threads == 512) ? 2 : 1;
+  return sizeof(typename CT<T>::t) == 8 ? (NX == 128 ? 2 : 3) : 1;
 }
 // z-pass threads per block for a tile of S columns of one row group (three
 // components): 24 S, one butterfly per thread in a radix-16 stage of the
@@ -293,7 +294,12 @@ __global__ void __launch_bounds__(xy_threads<T, NX>(), xy_min_blocks<T, NX>()) k
   // constant: loaded before the wait for the predecessor
   load_tables(twx, twy, posx, gtw, gpos, NX, NY, H, (sizeof(C) == 8 && NX == 128) ? tw0 : nullptr);
   pdl_wait();
-  if (skip && *(volatile const int*)skip) return;
+  // the stop flag is read by one thread (a read per warp makes its L2 line a
+  // queue) and tested after the first barrier behind the plane's loads
+  // (nothing is written before), and the first stage reads its twiddles from
+  // global memory: the loads wait neither for the flag nor for the tables
+  __shared__ int s_stop;
+  if (threadIdx.x == 0) s_stop = skip ? *(volatile const int*)skip : 0;
   const int c = blockIdx.x % 9, z = blockIdx.x / 9;
   const CI* src = reinterpret_cast<const CI*>(in + c * N + (long long)z * NY * NX);
   // row y, sample j (the real values 2j, 2j+1 as one complex sample)
@@ -304,20 +310,23 @@ __global__ void __launch_bounds__(xy_threads<T, NX>(), xy_min_blocks<T, NX>()) k
   };
   if constexpr (sizeof(C) == 8) {
     // FP32: the x transform touches shared memory twice per sample
-    __syncthreads();   // tables
     if constexpr (RowPlan<H>::NST == 2) {
       // first x stage straight from global memory (consecutive threads take
       // consecutive butterflies of a row: 64-byte row segments per warp access)
-      if constexpr (NX == 128)
+      if constexpr (NX == 128) {
+        __syncthreads();   // tables
+        if (s_stop) return;
         x_stage0_128<false, TPB>(tw0, gload, [&](int q, int e, C v) { buf[MF_AT(q * PX + e, NY * PX)] = v; });
-      else
+      } else {
         fft2::stage_io<C, H, NX, 0, false, NY, 1, PX, 0, 1, false>(
-            twx, [&](int q, int, int e) { return gload(q, e); },
+            gtw, [&](int q, int, int e) { return gload(q, e); },
             [&](int, int i, int, C v) { buf[MF_AT(i, NY * PX)] = v; });
+      }
       __syncthreads();
+      if (s_stop) return;
       x_last_split<T, NX, TPB>(buf, twx, [&](int y, int pos) { return buf[MF_AT(y * PX + pos, NY * PX)]; });
     } else {
-      x_last_split<T, NX, TPB>(buf, twx, gload);
+      x_last_split<T, NX, TPB>(buf, gtw, gload);
     }
   } else {
     // 16-byte types (FP64, double word) are arithmetic bound: the plane is
@@ -336,6 +345,7 @@ __global__ void __launch_bounds__(xy_threads<T, NX>(), xy_min_blocks<T, NX>()) k
       }
     }
     __syncthreads();
+    if (s_stop) return;
     fft2::forward<C, H, NX, NY, 1, PX, 0, 1>(buf, twx);
     constexpr int NP = H / 2 + 1;
     for (int idx = threadIdx.x; idx < NY * NP; idx += TPB) {
@@ -473,7 +483,13 @@ __global__ void __launch_bounds__(xy_threads<T, NX>(), xy_min_blocks<T, NX>()) k
   // constant: loaded before the wait for the predecessor
   load_tables(twx, twy, posx, gtw, gpos, NX, NY, H, (sizeof(C) == 8 && NX == 128) ? tw0 : nullptr);
   pdl_wait();
-  if (skip && *(volatile const int*)skip) return;
+  // (see k_xyf); alpha is needed at the end
+  __shared__ int s_stop;
+  __shared__ T s_alpha;
+  if (threadIdx.x == 0) {
+    s_stop = skip ? *(volatile const int*)skip : 0;
+    if (MODE == 3) s_alpha = (T)sc->alpha;
+  }
   const int c = blockIdx.x % 9, z = blockIdx.x / 9;
   if (MODE == 3) {
     // the residual plane is read only at the end: start pulling it into L2 now
@@ -483,9 +499,10 @@ __global__ void __launch_bounds__(xy_threads<T, NX>(), xy_min_blocks<T, NX>()) k
       asm volatile("prefetch.global.L2 [%0];" ::"l"(rp + 128 * i));
   }
   const C* src = spec + ((long long)c * nz + z) * NY * H;
-  __syncthreads();   // tables
-  // y: the first inverse stage reads the spectrum rows from global memory
+  // y: the first inverse stage reads the spectrum rows from global memory (no
+  // twiddles: the tables are ready with the barrier after it)
   fft2::inverse_in<C, NY, NY, H, 1, 1, 0, PX>(buf, twy, [&](int q, int e) { return src[MF_AT(e * H + q, NY * H)]; });
+  if (s_stop) return;
   if constexpr (sizeof(C) == 8) {
     // merge of each row's spectrum, fused with the first inverse x stage
     x_merge_first<T, NX, TPB>(buf, twx);
@@ -525,13 +542,16 @@ __global__ void __launch_bounds__(xy_threads<T, NX>(), xy_min_blocks<T, NX>()) k
     fadd(p);
     fadd(fmaf(v, v, -p));
   };
-  T alpha = (T)0;
-  if (MODE == 3) alpha = (T)sc->alpha;
-  // the output of sample (row y, j): y = G*(.) stored, or r -= alpha y
-  auto emit = [&](long long idx, C v) {
+  const T alpha = MODE == 3 ? s_alpha : (T)0;
+  // the output of sample (row y, j): y = G*(.) stored, or r -= alpha y (r
+  // loaded ahead by the caller)
+  auto fetch = [&](long long idx) {
+    if constexpr (MODE == 3) return dst[MF_AT(idx, NY * H)];
+    else return C();
+  };
+  auto emit = [&](long long idx, C v, C r) {
     idx = MF_AT(idx, NY * H);
     if constexpr (MODE == 3) {
-      C r = dst[idx];
       r.x -= alpha * v.x;
       r.y -= alpha * v.y;
       dst[idx] = r;
@@ -556,21 +576,28 @@ __global__ void __launch_bounds__(xy_threads<T, NX>(), xy_min_blocks<T, NX>()) k
   constexpr bool kDirect = sizeof(C) == 8 && RowPlan<H>::NST == 2 && (MODE != 3 || (M0 * 8) % 32 == 0);
   if constexpr (kDirect && NX == 128) {
     x_stage0_128<true, TPB>(tw0, [&](int q, int e) { return buf[MF_AT(q * PX + e, NY * PX)]; },
-                       [&](int q, int e, C v) { emit((long long)q * H + e, v); });
+                       [&](int q, int e, C v) { emit((long long)q * H + e, v, fetch((long long)q * H + e)); });
   } else if constexpr (kDirect) {
     // consecutive threads take consecutive butterflies of a row
-    fft2::stage_io<C, H, NX, 0, true, NY, 1, PX, 0, 1, false>(
-        twx, [&](int, int i, int) { return buf[MF_AT(i, NY * PX)]; },
-        [&](int q, int, int e, C v) { emit((long long)q * H + e, v); });
+    fft2::stage_rmw<C, H, NX, 0, true, NY, 1, PX, 0, 1, false>(
+        twx, [&](int, int i, int) { return buf[MF_AT(i, NY * PX)]; }, [&](int q, int e) { return fetch((long long)q * H + e); },
+        [&](int q, int e, C v, C r) { emit((long long)q * H + e, v, r); });
   } else {
     if constexpr (sizeof(C) == 8 && RowPlan<H>::NST == 2) {
       fft2::stage<C, H, NX, 0, true, NY, 1, PX, 0, 1, false>(buf, twx);
       __syncthreads();
     }
-#pragma unroll 8
-    for (int idx = threadIdx.x; idx < NY * H; idx += TPB) {
-      const int y = idx / H, j = idx - (idx / H) * H;
-      emit(idx, buf[MF_AT(y * PX + j, NY * PX)]);
+    constexpr int kAhead = MODE == 3 ? 4 : 1;   // values of r in flight per thread
+    for (int i0 = threadIdx.x; i0 < NY * H; i0 += kAhead * TPB) {
+      C r[kAhead];
+#pragma unroll
+      for (int k = 0; k < kAhead; ++k)
+        if (i0 + k * TPB < NY * H) r[k] = fetch(i0 + k * TPB);
+#pragma unroll
+      for (int k = 0; k < kAhead; ++k) {
+        const int idx = i0 + k * TPB;
+        if (idx < NY * H) emit(idx, buf[MF_AT((idx / H) * PX + idx % H, NY * PX)], r[k]);
+      }
     }
   }
   if (sizeof(TI) == 4) acc = (double)fs + (double)fc;
@@ -648,7 +675,8 @@ __global__ void __launch_bounds__(z_threads(S_), z_min_blocks<T>(S_, MODE)) k_zp
     xiz[i] = ((NZ % 2 == 0) && (2 * kz == NZ)) ? (TX)NAN : (TX)kzs * ((TX)1 / (TX)NZ);
   }
   pdl_wait();
-  if (a.skip && *(volatile const int*)a.skip) return;
+  __shared__ int s_stop;   // tested after the first barrier (see k_xyf)
+  if (threadIdx.x == 0) s_stop = a.skip ? *(volatile const int*)a.skip : 0;
   const int H = a.nx / 2;
   const int ncol = a.ny * H;
   const int ntile = ncol / S;
@@ -661,30 +689,32 @@ __global__ void __launch_bounds__(z_threads(S_), z_min_blocks<T>(S_, MODE)) k_zp
   auto gidx = [&](int q, int z) {
     return MF_AT(goff + ((long long)(q / S) * NZ + z) * ncol + (q % S), 9LL * NZ * ncol) - goff;
   };
-  if (MODE == 0 && a.lin) {
-    // the null-frequency coefficient of each component of the row group is
-    // the sum over z of its planes' (kx, ky) = (0, 0) coefficients: read
-    // here, before the transform overwrites them, by the block holding that
-    // column (one warp per component, summed in FP64)
-    int sdc = -1;
-    for (int s = 0; s < S; ++s) {
-      const int col = col0 + s, row = col / H, slot = col - row * H;
-      if (a.xk[slot] == 0 && a.yk[row] == 0) sdc = s;
-    }
-    if (sdc >= 0 && threadIdx.x < 96) {
-      const int cl = threadIdx.x >> 5, lane = threadIdx.x & 31;
-      double sum = 0.0;
-      for (int z = lane; z < NZ; z += 32) sum += (double)gsp[gidx(cl * S + sdc, z)].x;
-      for (int o = 16; o > 0; o >>= 1) sum += __shfl_xor_sync(0xffffffffu, sum, o);
-      if (lane == 0) a.lin[3 * g + cl] += *a.lin_alpha * (sum / (double)a.N);
+  // the null-frequency coefficient of each component of the row group is the
+  // sum over z of its planes' (kx, ky) = (0, 0) coefficients, the first column
+  // (digit reversal keeps 0): read here, before the transform overwrites them,
+  // by the block holding that column (one warp per component), summed in FP64
+  // at the end, off the transform's path
+  // (each value waits in shared memory for the thread that put it there)
+  constexpr int kDc = MODE == 0 ? NZ : 1;
+  __shared__ float s_dc[3][kDc];
+  __shared__ double s_lin[3], s_lin_alpha[3];
+  if (MODE == 0 && a.lin && col0 == 0 && threadIdx.x < 96) {
+    const int cl = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    for (int z = lane; z < kDc; z += 32) s_dc[cl][z] = (float)gsp[gidx(cl * S, z)].x;
+    if (lane == 0) {
+      s_lin_alpha[cl] = *a.lin_alpha;
+      s_lin[cl] = a.lin[3 * g + cl];
     }
   }
-  __syncthreads();
   if constexpr (NST > 1) {
-    // first forward stage: global -> registers -> shared
+    // first forward stage: global -> registers -> shared (FP32: twiddles from
+    // global memory, no barrier for the tables; the 16-byte types would hold
+    // the twiddles they load ahead in registers)
+    if constexpr (!Sh::E8) __syncthreads();
     fft2::stage_io<C, NZ, NZ, 0, false, 3 * S, S, CP, 1, ZS, true>(
-        twz, [&](int q, int, int z) { return gsp[gidx(q, z)]; }, [&](int, int i, int, C v) { buf[MF_AT(i, 3 * CP)] = v; });
+        Sh::E8 ? gtwz : twz, [&](int q, int, int z) { return gsp[gidx(q, z)]; }, [&](int, int i, int, C v) { buf[MF_AT(i, 3 * CP)] = v; });
     __syncthreads();
+    if (s_stop) return;
     if constexpr (NST > 2) {
       fft2::stage<C, NZ, NZ, 1, false, 3 * S, S, CP, 1, ZS, true>(buf, twz);
       __syncthreads();
@@ -735,7 +765,7 @@ __global__ void __launch_bounds__(z_threads(S_), z_min_blocks<T>(S_, MODE)) k_zp
       v2 = cmake(q.x * xi2, q.y * xi2);
     }
   };
-  if constexpr (sizeof(C) == 8 && NST > 1) {
+  if constexpr (sizeof(C) == 8 && NST > 1 && RL <= 8) {
     // FP32: last forward stage, G-hat-star and first inverse stage in
     // registers (three components of RL positions of one column per thread)
     constexpr int NB = NZ / RL;
@@ -766,15 +796,17 @@ __global__ void __launch_bounds__(z_threads(S_), z_min_blocks<T>(S_, MODE)) k_zp
   } else {
     // 16-byte types (FP64, double word): registers are scarcer, so the last
     // forward stage, G-hat-star and the first inverse stage are separate
-    // passes over shared memory.  So they are for nz = 16 in FP32, one radix-16
-    // stage: in registers it left eight threads a block with all the work
-    // (three transforms and sixteen G-hat-star evaluations each, 14 us a launch)
+    // passes over shared memory.  So they are in FP32 where the last stage is
+    // radix 16: for nz = 16, one stage, registers left eight threads a block
+    // with all the work (14 us a launch); for nz = 256 three butterflies of 16
+    // do not fit the 64 registers of the tile's occupancy (0.9 KB of spills)
     if constexpr (NST == 1) {
       for (int idx = threadIdx.x; idx < 3 * NZ * S; idx += kZThreads) {
         const int s2 = idx % S, cz = idx / S, cl = cz / NZ, z = cz - cl * NZ;
         buf[cl * CP + z * ZS + s2] = gsp[gidx(cl * S + s2, z)];
       }
       __syncthreads();
+      if (s_stop) return;
     }
     fft2::stage<C, NZ, NZ, NST - 1, false, 3 * S, S, CP, 1, ZS, true>(buf, twz);
     __syncthreads();
@@ -802,6 +834,13 @@ __global__ void __launch_bounds__(z_threads(S_), z_min_blocks<T>(S_, MODE)) k_zp
     // last inverse stage: shared -> registers -> global
     fft2::stage_io<C, NZ, NZ, 0, true, 3 * S, S, CP, 1, ZS, true>(
         twz, [&](int, int i, int) { return buf[MF_AT(i, 3 * CP)]; }, [&](int q, int, int z, C v) { gsp[gidx(q, z)] = v; });
+  }
+  if (MODE == 0 && a.lin && col0 == 0 && threadIdx.x < 96) {
+    const int cl = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    double sum = 0.0;
+    for (int z = lane; z < kDc; z += 32) sum += (double)s_dc[cl][z];
+    for (int o = 16; o > 0; o >>= 1) sum += __shfl_xor_sync(0xffffffffu, sum, o);
+    if (lane == 0) a.lin[3 * g + cl] = s_lin[cl] + s_lin_alpha[cl] * (sum / (double)a.N);
   }
 }
 

@@ -142,26 +142,31 @@ __global__ void __launch_bounds__(512, xy_min_blocks<T>()) k_xyf(const T* __rest
   int* posx = reinterpret_cast<int*>(twy + ny);
   load_tables(twx, twy, posx, a);   // constant: before the wait for the predecessor
   pdl_wait();
-  if (a.skip && *(volatile const int*)a.skip) return;
+  // the stop flag is read by one thread (a read per warp makes its L2 line a
+  // queue) and tested after the first barrier behind the plane's loads
+  // (nothing is written before), and the first pass reads its twiddles from
+  // global memory: the loads wait neither for the flag nor for the tables
+  __shared__ int s_stop;
+  if (threadIdx.x == 0) s_stop = a.skip ? *(volatile const int*)a.skip : 0;
   const int c = blockIdx.x % 9, z = blockIdx.x / 9;
   const T* src = in + c * a.N + (long long)z * ny * nx;
   const int ext = hy * PX, half = hy * nx;
   (void)ext;
-  __syncthreads();   // tables
   // x: rows q and q + ny/2 as one complex row; the first pass reads the two
   // real rows along themselves
-  pass<C, false, false>(a.px, 0, hy, a.dhy, twx,
+  pass<C, false, false>(a.px, 0, hy, a.dhy, reinterpret_cast<const C*>(a.twx),
                         [&](int q, int e) {
                           const int i = MF_AT(q * nx + e, half);
                           return cmake(src[i], src[i + half]);
                         },
                         [&](int q, int e, C v) { buf[MF_AT(q * PX + e, ext)] = v; });
+  __syncthreads();
+  if (s_stop) return;
   for (int g = 1; g < a.px.npass; ++g) {
-    __syncthreads();
     pass<C, false, true>(a.px, g, hy, a.dhy, twx, [&](int q, int e) { return buf[MF_AT(q * PX + e, ext)]; },
                          [&](int q, int e, C v) { buf[MF_AT(q * PX + e, ext)] = v; });
+    __syncthreads();
   }
-  __syncthreads();
   // split the packed rows into the spectra of rows q and q + ny/2, and apply
   // the first (radix-2) stage of the y transform, which combines those two
   for (int idx = threadIdx.x; idx < hy * hx; idx += blockDim.x) {
@@ -209,7 +214,13 @@ __global__ void __launch_bounds__(512, xy_min_blocks<T>()) k_xyi(const typename 
   int* posx = reinterpret_cast<int*>(twy + ny);
   load_tables(twx, twy, posx, a);   // constant: before the wait for the predecessor
   pdl_wait();
-  if (a.skip && *(volatile const int*)a.skip) return;
+  // (see k_xyf); alpha is needed at the end
+  __shared__ int s_stop;
+  __shared__ T s_alpha;
+  if (threadIdx.x == 0) {
+    s_stop = a.skip ? *(volatile const int*)a.skip : 0;
+    if (MODE == 3) s_alpha = (T)sc->alpha;
+  }
   const int c = blockIdx.x % 9, z = blockIdx.x / 9;
   const int ext = hy * PX, half = hy * nx;
   (void)ext;
@@ -221,16 +232,17 @@ __global__ void __launch_bounds__(512, xy_min_blocks<T>()) k_xyi(const typename 
     for (int i = threadIdx.x * 128; i < ny * nx * (int)sizeof(T); i += blockDim.x * 128)
       asm volatile("prefetch.global.L2 [%0];" ::"l"(rp + i));
   }
-  __syncthreads();   // tables
   // y: the first inverse pass reads the spectrum
-  pass<C, true, true>(a.py, a.py.npass - 1, nx, a.dnx, twy, [&](int q, int e) { return src[MF_AT(e * nx + q, half)]; },
+  pass<C, true, true>(a.py, a.py.npass - 1, nx, a.dnx, reinterpret_cast<const C*>(a.twy),
+                      [&](int q, int e) { return src[MF_AT(e * nx + q, half)]; },
                       [&](int q, int e, C v) { buf[MF_AT(e * PX + q, ext)] = v; });
+  __syncthreads();
+  if (s_stop) return;
   for (int g = a.py.npass - 2; g >= 0; --g) {
-    __syncthreads();
     pass<C, true, true>(a.py, g, nx, a.dnx, twy, [&](int q, int e) { return buf[MF_AT(e * PX + q, ext)]; },
                         [&](int q, int e, C v) { buf[MF_AT(e * PX + q, ext)] = v; });
+    __syncthreads();
   }
-  __syncthreads();
   for (int idx = threadIdx.x; idx < hy * hx; idx += blockDim.x) {
     const int k = fdiv(idx, a.dhy), q = idx - k * hy;
     C* row = buf + MF_AT(q * PX, ext - nx + 1);
@@ -276,17 +288,28 @@ __global__ void __launch_bounds__(512, xy_min_blocks<T>()) k_xyi(const typename 
         acc += (double)v * (double)v;
       }
     };
-    const T alpha = (T)sc->alpha;
-#pragma unroll 4
-    for (int idx = threadIdx.x; idx < half; idx += blockDim.x) {
-      const int q = fdiv(idx, a.dnx);
-      const int i = MF_AT(idx, half);
-      const C v = buf[MF_AT(q * PX + idx - q * nx, ext)];
-      const T r0 = dst[i] - alpha * v.x, r1 = dst[i + half] - alpha * v.y;
-      dst[i] = r0;
-      dst[i + half] = r1;
-      add2(r0);
-      add2(r1);
+    const T alpha = s_alpha;
+    constexpr int kAhead = 4;   // pairs of r in flight per thread
+    for (int i0 = threadIdx.x; i0 < half; i0 += kAhead * blockDim.x) {
+      T ra[kAhead], rb[kAhead];
+#pragma unroll
+      for (int k = 0; k < kAhead; ++k) {
+        const int i = i0 + k * blockDim.x;
+        if (i < half) { ra[k] = dst[i]; rb[k] = dst[i + half]; }
+      }
+#pragma unroll
+      for (int k = 0; k < kAhead; ++k) {
+        const int i = i0 + k * blockDim.x;
+        if (i < half) {
+          const int q = fdiv(i, a.dnx);
+          const C v = buf[MF_AT(q * PX + i - q * nx, ext)];
+          const T r0 = ra[k] - alpha * v.x, r1 = rb[k] - alpha * v.y;
+          dst[i] = r0;
+          dst[i + half] = r1;
+          add2(r0);
+          add2(r1);
+        }
+      }
     }
     if (sizeof(T) == 4) acc = (double)fs + (double)fc;
     for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
@@ -340,7 +363,8 @@ __global__ void __launch_bounds__(256) k_zp(typename CT<T>::t* __restrict__ spec
     xiz[i] = (T)((2 * kz < nz) ? kz : kz - nz) / (T)nz;
   }
   pdl_wait();
-  if (a.skip && *(volatile const int*)a.skip) return;
+  __shared__ int s_stop;   // tested after the first barrier (see k_xyf)
+  if (threadIdx.x == 0) s_stop = a.skip ? *(volatile const int*)a.skip : 0;
   const int ntile = (ncol + S - 1) / S;
   const int g = blockIdx.x / ntile;
   const int col0 = (blockIdx.x - g * ntile) * S;
@@ -361,9 +385,9 @@ __global__ void __launch_bounds__(256) k_zp(typename CT<T>::t* __restrict__ spec
   auto sst = [&](int q, int z, C v) { buf[MF_AT((q / S) * CP + z * ZS + q % S, ext)] = v; };
   constexpr int NSEQ = 3 * S;
   const FastDiv dseq = a.dseq;
-  __syncthreads();   // tables
-  pass<C, false, true>(a.pz, 0, NSEQ, dseq, twz, gld, sst);
+  pass<C, false, true>(a.pz, 0, NSEQ, dseq, gtwz, gld, sst);
   __syncthreads();
+  if (s_stop) return;
   for (int p = 1; p < a.pz.npass; ++p) {
     pass<C, false, true>(a.pz, p, NSEQ, dseq, twz, sld, sst);
     __syncthreads();

@@ -39,27 +39,32 @@ __device__ __forceinline__ double2 io_out(dwc v) { return to_double2(v); }
 constexpr int kThreads = 256;
 // x-y kernels: 16-byte elements (FP64, double word) hold one 128 x 128 plane
 // in 133 KB of shared memory, one block per SM, so they run twice the
-// threads; FP32 128 x 128 planes (66 KB) run two blocks of 512 threads per
+// threads; planes up to 64 x 64 run three blocks of 256, of 96 x 96 two of
+// 512, whose barriers and load phases overlap (double-word residual against
+// one block of 512: 32^3 31 -> 23 us, 48^3 69 -> 49, 64^3 94 -> 80, 96^3 341
+// -> 310).  FP32 128 x 128 planes (66 KB) run two blocks of 512 threads per
 // SM at 64 registers a thread (about 1% faster than three blocks of 256 on
 // the GB300), other FP32 planes blocks of 256
 constexpr int kXY128Threads = 512;
 template <typename T, int NX> __host__ __device__ constexpr int xy_threads() {
-  return sizeof(typename CT<T>::t) == 16 ? 512 : (NX == 128 ? kXY128Threads : 256);
+  if (sizeof(typename CT<T>::t) == 16) return NX <= 64 ? 256 : 512;
+  return NX == 128 ? kXY128Threads : 256;
 }
-// resident blocks per SM the register allocation of an FP32 x-y kernel is
-// held to: two of 512 threads (128 x 128 planes, 64 registers a thread),
-// three of 256
+// resident blocks per SM the register allocation of an x-y kernel is held to
 template <typename T, int NX> __host__ __device__ constexpr int xy_min_blocks() {
-  return sizeof(typename CT<T>::t) == 8 ? (NX == 128 ? 2 : 3) : 1;
+  if (sizeof(typename CT<T>::t) == 16) return NX <= 64 ? 3 : (NX == 96 ? 2 : 1);
+  return NX == 128 ? 2 : 3;
 }
 // z-pass threads per block for a tile of S columns of one row group (three
 // components): 24 S, one butterfly per thread in a radix-16 stage of the
 // 128-point transform and two in its radix-8 stage (3 x S x 128/R)
 __host__ __device__ constexpr int z_threads(int S) { return 24 * S; }
 // resident z-pass blocks per SM the register allocation is held to: five
-// blocks of 192 threads for the FP32 operator pass (S = 8, MODE 0), else what
-// the compiler chooses
+// blocks of 192 threads for the FP32 operator pass (S = 8, MODE 0), three for
+// the double-word residual (112 registers instead of 138: 128^3 residual 698
+// -> 686 us), else what the compiler chooses
 template <typename T> __host__ __device__ constexpr int z_min_blocks(int S, int mode) {
+  if (S == 8 && std::is_same<T, dw>::value) return 3;
   return (sizeof(typename CT<T>::t) == 8 && S == 8 && mode == 0) ? 5 : 1;
 }
 

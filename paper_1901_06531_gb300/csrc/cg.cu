@@ -25,25 +25,6 @@ namespace {
 constexpr int kThreads = 256;
 constexpr int kTangentBlocks = 152 * 8;   // rows of the table of partial sums the callers provide
 
-template <int NC>
-__device__ __forceinline__ void block_sum_cg(double (&v)[NC], double* out) {
-  __shared__ double red[NC][32];
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-#pragma unroll
-  for (int c = 0; c < NC; ++c) {
-    double s = v[c];
-    for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
-    if (lane == 0) red[c][warp] = s;
-  }
-  __syncthreads();
-  if (threadIdx.x < NC) {
-    double s = 0.0;
-    for (int w = 0; w < (int)(blockDim.x >> 5); ++w) s += red[threadIdx.x][w];
-    out[threadIdx.x] = s;
-  }
-  __syncthreads();
-}
-
 // Per-thread dot-product accumulator: exact FP32 products (two-product by FMA)
 // summed with Neumaier compensation in FP32; the thread totals are then
 // combined in FP64.  FP64 arithmetic per element would cost as much as the
@@ -165,8 +146,9 @@ __global__ void __launch_bounds__(kThreads, TAN == 0 ? 2 : (CG ? 4 : 5)) k_tange
                                                       TangentArgs ta, T* __restrict__ t, long long N,
                                                       double* __restrict__ partials, Scalars* sc) {
   static_assert(!FIN || CG, "the fused finish belongs to the CG pass");
-  __shared__ double tot[1];
+  __shared__ double red[32];
   T beta = (T)0, alpha = (T)0;
+  double rr = 0.0;   // thread 0
   pdl_wait();
   bool first = false;   // first CG iteration: p = r, x = 0 (neither previous vector is read)
   if (CG) {
@@ -178,6 +160,7 @@ __global__ void __launch_bounds__(kThreads, TAN == 0 ? 2 : (CG ? 4 : 5)) k_tange
     if (threadIdx.x == 0) {
       const int stop = *(volatile const int*)&sc->stop, its = *(volatile const int*)&sc->its;
       const double b = *(volatile const double*)&sc->beta, a = *(volatile const double*)&sc->alpha;
+      if (FIN) rr = *(volatile const double*)&sc->rr;
       s_stop = stop;
       s_its = its;
       s_beta = (T)b;
@@ -269,12 +252,11 @@ __global__ void __launch_bounds__(kThreads, TAN == 0 ? 2 : (CG ? 4 : 5)) k_tange
     for (long long v = v0; v < N; v += dv) voxel(v, std::false_type{});
   }
   if (partials) {
-    double acc[1] = {sizeof(T) == 4 ? acc32.value() : acc64};
-    block_sum_cg<1>(acc, tot);
-    if (threadIdx.x == 0) partials[blockIdx.x] = tot[0];
+    const double acc = block_total(sizeof(T) == 4 ? acc32.value() : acc64, red);
+    if (threadIdx.x == 0) partials[blockIdx.x] = acc;
     if constexpr (FIN) {
       double pAp;
-      if (last_block_total(partials, &sc->arrive, &pAp) && threadIdx.x == 0) cg_finish_alpha(pAp, sc);
+      if (last_block_total(partials, &sc->arrive, &pAp) && threadIdx.x == 0) cg_finish_alpha(pAp, rr, sc);
     }
   }
 }
@@ -297,8 +279,10 @@ __global__ void __launch_bounds__(kThreads) k_fin_beta(const double* __restrict_
                                                        Scalars* sc) {
   __shared__ double shm[kThreads];
   if (*(volatile const int*)&sc->stop) return;
+  CgScalars cs;
+  cs.load(sc);
   const double rr = col_sum(partials, n, shm);
-  if (threadIdx.x == 0) cg_finish_beta(rr, sc);
+  if (threadIdx.x == 0) cg_finish_beta(rr, cs, sc);
 }
 
 template <typename T>

@@ -215,34 +215,48 @@ struct Scalars {
   unsigned arrive;    // blocks of the current pass that have stored their partial sum
 };
 
-// Grid-wide sum finished by the last block to arrive: every block has stored
-// its partial sum in partials[blockIdx.x] (thread 0 wrote it); thread 0
-// publishes it and counts the block in *arrive.  The block that arrives last
-// adds all partials in a fixed order, leaves the total in *total (read by
-// every thread), resets the counter and returns true; the others return
+// Sum of one value per thread over the block (whole warps, at most 32; red:
+// 32 shared doubles), in thread 0.  The warps' sums are combined in log2 of
+// their number of steps: each dependent FP64 addition is a step of the
+// latency chain that ends a CG kernel.
+__device__ __forceinline__ double block_total(double v, double* red) {
+  const int lane = threadIdx.x & 31, nw = blockDim.x >> 5;
+  for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+  if (lane == 0) red[threadIdx.x >> 5] = v;
+  __syncthreads();
+  v = 0.0;
+  if (threadIdx.x < 32) {
+    v = lane < nw ? red[lane] : 0.0;
+    for (int o = nw > 16 ? 16 : (nw > 8 ? 8 : (nw > 4 ? 4 : (nw > 2 ? 2 : 1))); o > 0; o >>= 1)
+      v += __shfl_xor_sync(0xffffffffu, v, o);
+  }
+  return v;
+}
+
+// Grid-wide sum finished by the last block to arrive: every block's thread 0
+// has stored its partial sum in partials[blockIdx.x]; here it counts the
+// block in *arrive (one acquire-release operation publishes the partial and,
+// in the last block, orders the reads of the others behind it).  The block
+// that arrives last adds all partials in a fixed order, leaves the total in
+// *total (thread 0), resets the counter and returns true; the others return
 // false.  No block waits on another.
 __device__ __forceinline__ bool last_block_total(const double* partials, unsigned* arrive, double* total) {
   __shared__ unsigned s_last;
   __shared__ double s_red[32];
   if (threadIdx.x == 0) {
-    __threadfence();
-    s_last = (atomicAdd(arrive, 1u) == gridDim.x - 1) ? 1u : 0u;
+    unsigned before;
+    asm volatile("atom.add.acq_rel.gpu.global.u32 %0, [%1], 1;" : "=r"(before) : "l"(arrive) : "memory");
+    s_last = (before == gridDim.x - 1) ? 1u : 0u;
   }
   __syncthreads();
   if (!s_last) return false;
-  __threadfence();
   double s = 0.0;
   for (unsigned b = threadIdx.x; b < gridDim.x; b += blockDim.x) s += __ldcg(partials + b);
-  for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
-  if ((threadIdx.x & 31) == 0) s_red[threadIdx.x >> 5] = s;
-  __syncthreads();
-  if (threadIdx.x < 32) {
-    double t = (threadIdx.x < (blockDim.x >> 5)) ? s_red[threadIdx.x] : 0.0;
-    for (int o = 16; o > 0; o >>= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
-    if (threadIdx.x == 0) { s_red[0] = t; *arrive = 0u; }
+  s = block_total(s, s_red);
+  if (threadIdx.x == 0) {
+    *total = s;
+    *arrive = 0u;
   }
-  __syncthreads();
-  *total = s_red[0];
   return true;
 }
 
@@ -251,24 +265,40 @@ __device__ __forceinline__ bool last_block_total(const double* partials, unsigne
 #define MF_FLAG_NONFINITE 4
 #define MF_FLAG_TIMEOUT 8     // a bounded device-side wait gave up
 
+// The scalars the updates below need, as the previous kernel left them: the
+// fused passes read them when they start, off the chain at their end.
+struct CgScalars {
+  double rr, thr2N;
+  int flags, its, max_its;
+  __device__ __forceinline__ void load(const Scalars* sc) {
+    rr = sc->rr;
+    thr2N = sc->thr2N;
+    flags = sc->flags;
+    its = sc->its;
+    max_its = sc->max_its;
+  }
+};
+
 // CG scalar updates after the curvature p.Ap and after the new r.r (shared by
 // the one-block finishing kernels and the last blocks of fused passes).
-__device__ __forceinline__ void cg_finish_alpha(double pAp, Scalars* sc) {
+__device__ __forceinline__ void cg_finish_alpha(double pAp, double rr, Scalars* sc) {
   sc->pAp = pAp;
   if (!(pAp > 0.0) || !isfinite(pAp)) {
     sc->flags |= MF_FLAG_BREAKDOWN;
     sc->alpha = 0.0;
     sc->stop = 1;
   } else {
-    sc->alpha = sc->rr / pAp;
+    sc->alpha = rr / pAp;
   }
 }
 
-__device__ __forceinline__ void cg_finish_beta(double rr, Scalars* sc) {
-  if (!isfinite(rr)) sc->flags |= MF_FLAG_NONFINITE;
-  sc->beta = rr / sc->rr;
+__device__ __forceinline__ void cg_finish_beta(double rr, const CgScalars& b, Scalars* sc) {
+  int flags = b.flags;
+  if (!isfinite(rr)) sc->flags = flags = flags | MF_FLAG_NONFINITE;
+  sc->beta = rr / b.rr;
   sc->rr = rr;
-  sc->done = (rr <= sc->thr2N) ? 1 : 0;
-  sc->its += 1;
-  sc->stop = (sc->done || sc->flags || sc->its >= sc->max_its) ? 1 : 0;
+  const int done = (rr <= b.thr2N) ? 1 : 0;
+  sc->done = done;
+  sc->its = b.its + 1;
+  sc->stop = (done || flags || b.its + 1 >= b.max_its) ? 1 : 0;
 }

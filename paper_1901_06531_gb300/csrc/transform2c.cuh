@@ -374,7 +374,11 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(clu::kCThreads, 4)
     }
     if (MODE == 3 && fin) {
       double rr;
-      if (last_block_total(partials, &sc->arrive, &rr) && threadIdx.x == 0) cg_finish_beta(rr, sc);
+      if (last_block_total(partials, &sc->arrive, &rr) && threadIdx.x == 0) {
+        CgScalars cs;
+        cs.load(sc);
+        cg_finish_beta(rr, cs, sc);
+      }
     }
   }
 }

@@ -217,9 +217,13 @@ __global__ void __launch_bounds__(512, xy_min_blocks<T>()) k_xyi(const typename 
   // (see k_xyf); alpha is needed at the end
   __shared__ int s_stop;
   __shared__ T s_alpha;
+  __shared__ CgScalars s_cg;
   if (threadIdx.x == 0) {
     s_stop = a.skip ? *(volatile const int*)a.skip : 0;
-    if (MODE == 3) s_alpha = (T)sc->alpha;
+    if (MODE == 3) {
+      s_alpha = (T)sc->alpha;
+      if (a.fin) s_cg.load(sc);
+    }
   }
   const int c = blockIdx.x % 9, z = blockIdx.x / 9;
   const int ext = hy * PX, half = hy * nx;
@@ -312,17 +316,11 @@ __global__ void __launch_bounds__(512, xy_min_blocks<T>()) k_xyi(const typename 
       }
     }
     if (sizeof(T) == 4) acc = (double)fs + (double)fc;
-    for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
-    if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = acc;
-    __syncthreads();
-    if (threadIdx.x < 32) {
-      double s = (threadIdx.x < (blockDim.x >> 5)) ? red[threadIdx.x] : 0.0;
-      for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
-      if (threadIdx.x == 0) partials[blockIdx.x] = s;
-    }
+    acc = block_total(acc, red);
+    if (threadIdx.x == 0) partials[blockIdx.x] = acc;
     if (a.fin) {
       double rr;
-      if (last_block_total(partials, &sc->arrive, &rr) && threadIdx.x == 0) cg_finish_beta(rr, sc);
+      if (last_block_total(partials, &sc->arrive, &rr) && threadIdx.x == 0) cg_finish_beta(rr, s_cg, sc);
     }
   } else {
     pass<C, true, false>(a.px, 0, hy, a.dhy, twx, sload, [&](int q, int e, C v) {

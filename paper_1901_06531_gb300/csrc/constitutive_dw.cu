@@ -200,7 +200,7 @@ __global__ void __launch_bounds__(kThreads, 2) k_constitutive_dw(double* __restr
   bool bad = false;
   __shared__ PredCoef pk_s;   // the predictor's coefficients (PRED), read from shared memory at each use
   if constexpr (PRED) {
-    if (threadIdx.x == 0) pk_s = pred_coef(pa, sc);
+    pred_coef_block(pa, sc, &pk_s);
     __syncthreads();
   }
   volatile PredCoef& pk = pk_s;

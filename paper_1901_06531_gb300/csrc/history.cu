@@ -385,32 +385,38 @@ __global__ void k_predictor_hist(double* __restrict__ F, PredArgs pa, long long 
                                  bool after_update) {
   const HistState* hs = pa.hs;
   const long long v0 = blockIdx.x * (long long)blockDim.x + threadIdx.x, dv = (long long)gridDim.x * blockDim.x;
+  __shared__ PredCoef ks;   // coefficients taken once per block: FP64 arithmetic per thread would cost more than the pass
   if (after_update || pa.kind == 0) {
-    // the strain-controlled components only
-    const PredCoef k = pred_coef(pa, sc);
+    // the strain-controlled components only (N is even: two values per step)
+    __shared__ int on[9];
+    if (threadIdx.x < 9) {
+      const int c = threadIdx.x;
+      on[c] = !hs->mask[c];
+      if (after_update) ks.sh[c] = hs->target[c] - sc->meanF_new[c];
+    }
+    if (!after_update) pred_coef_block(pa, sc, &ks);
+    __syncthreads();
     for (int c = 0; c < 9; ++c) {
-      if (hs->mask[c]) continue;
-      const double shift = after_update ? hs->target[c] - sc->meanF_new[c] : k.sh[c];
-      for (long long v = v0; v < N; v += dv) F[c * N + v] += shift;
+      if (!on[c]) continue;
+      const double shift = ks.sh[c];
+      double2* F2 = reinterpret_cast<double2*>(F + c * N);
+      for (long long v = v0; v < N / 2; v += dv) {
+        double2 f = F2[v];
+        f.x += shift;
+        f.y += shift;
+        F2[v] = f;
+      }
     }
     return;
   }
   // a flat pass over the 9N values, two per step (16-byte accesses where N
   // is even; a pair never spans two components then), the coefficients in
   // shared memory; the form of predict.cuh
-  __shared__ double sh[9];
-  __shared__ double w12[2];
-  __shared__ int dsts;
-  if (threadIdx.x == 0) {
-    const PredCoef k = pred_coef(pa, sc);
-    for (int c = 0; c < 9; ++c) sh[c] = k.sh[c];
-    w12[0] = k.v1;
-    w12[1] = k.v2;
-    dsts = k.dst;
-  }
+  pred_coef_block(pa, sc, &ks);
   __syncthreads();
-  const double v1 = w12[0], v2 = w12[1];
-  const int dst = dsts;
+  const double* sh = ks.sh;
+  const double v1 = ks.v1, v2 = ks.v2;
+  const int dst = ks.dst;
   double* __restrict__ A = pa.A;
   double* __restrict__ B = pa.B;
   auto one = [&](double f, double a, double b, int c) {

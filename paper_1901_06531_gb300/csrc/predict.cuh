@@ -26,28 +26,28 @@ struct PredCoef {
   int dst;
 };
 
-// The coefficients of the step that k_step_begin prepared; sc->meanF: the
-// averages of the current (last converged) F.
-__device__ __forceinline__ PredCoef pred_coef(const PredArgs& pa, const Scalars* sc) {
+// The coefficients of the step that k_step_begin prepared, by the first nine
+// threads of a block into shared memory (the caller synchronises); sc->meanF:
+// the averages of the current (last converged) F.
+__device__ __forceinline__ void pred_coef_block(const PredArgs& pa, const Scalars* sc, PredCoef* k) {
+  if (threadIdx.x >= 9) return;
   const HistState* hs = pa.hs;
-  PredCoef k;
-  k.v1 = 0.0;
-  k.v2 = 0.0;
-  k.dst = -1;
+  const int c = threadIdx.x;
   if (pa.kind == 2) {
     const bool qx = hs->extrapolated && hs->quad;
-    k.v1 = qx ? hs->w[1] : 0.0;
-    k.v2 = qx ? hs->w[2] : 0.0;
-    k.dst = hs->dst;
-    for (int c = 0; c < 9; ++c) k.sh[c] = hs->mask[c] ? 0.0 : hs->target[c] - (qx ? hs->pmean[c] : sc->meanF[c]);
+    k->sh[c] = hs->mask[c] ? 0.0 : hs->target[c] - (qx ? hs->pmean[c] : sc->meanF[c]);
+    if (c == 0) {
+      k->v1 = qx ? hs->w[1] : 0.0;
+      k->v2 = qx ? hs->w[2] : 0.0;
+      k->dst = hs->dst;
+    }
   } else {
     const double a = (pa.kind == 1 && hs->extrapolated) ? hs->alpha : 0.0;
-    if (pa.kind == 1) {
-      k.v1 = -a;
-      k.dst = 0;
+    k->sh[c] = hs->mask[c] ? 0.0 : hs->target[c] - (sc->meanF[c] + a * (sc->meanF[c] - hs->fmean2[c]));
+    if (c == 0) {
+      k->v1 = pa.kind == 1 ? -a : 0.0;
+      k->v2 = 0.0;
+      k->dst = pa.kind == 1 ? 0 : -1;
     }
-    for (int c = 0; c < 9; ++c)
-      k.sh[c] = hs->mask[c] ? 0.0 : hs->target[c] - (sc->meanF[c] + a * (sc->meanF[c] - hs->fmean2[c]));
   }
-  return k;
 }

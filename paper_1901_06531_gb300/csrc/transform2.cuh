@@ -279,6 +279,18 @@ __device__ __forceinline__ void x_merge_first(typename CT<T>::t* buf, const type
   }
 }
 
+// Row that the j-th group of lanes takes in the first (last inverse) x stage
+// of an FP32 plane, whose NB = H / radix butterflies per row sit NB consecutive
+// elements apart: rows whose NB-element groups tile the 16 banks (pitch H + 1),
+// so that a half-warp needs one wavefront instead of 2 to 4 with consecutive
+// rows (NB = 3 for 48 and 96, 4 for 64; 128: x_stage0_128).
+template <int NX> __device__ __forceinline__ int x_row(int j) {
+  if (NX == 48) return (11 * j) % 48;
+  if (NX == 64) return 4 * (j % 16) + j / 16;
+  if (NX == 96) return 3 * (j % 32) + j / 32;
+  return j;
+}
+
 // ------------------------------------------------------------------ forward
 template <typename T, int NX>
 __global__ void __launch_bounds__(xy_threads<T, NX>(), xy_min_blocks<T, NX>()) k_xyf(const typename IOT<T>::t* __restrict__ in,
@@ -324,8 +336,8 @@ __global__ void __launch_bounds__(xy_threads<T, NX>(), xy_min_blocks<T, NX>()) k
         x_stage0_128<false, TPB>(tw0, gload, [&](int q, int e, C v) { buf[MF_AT(q * PX + e, NY * PX)] = v; });
       } else {
         fft2::stage_io<C, H, NX, 0, false, NY, 1, PX, 0, 1, false>(
-            gtw, [&](int q, int, int e) { return gload(q, e); },
-            [&](int, int i, int, C v) { buf[MF_AT(i, NY * PX)] = v; });
+            gtw, [&](int q, int, int e) { return gload(x_row<NX>(q), e); },
+            [&](int q, int, int e, C v) { buf[MF_AT(x_row<NX>(q) * PX + e, NY * PX)] = v; });
       }
       __syncthreads();
       if (s_stop) return;
@@ -589,11 +601,14 @@ __global__ void __launch_bounds__(xy_threads<T, NX>(), xy_min_blocks<T, NX>()) k
   } else if constexpr (kDirect) {
     // consecutive threads take consecutive butterflies of a row
     fft2::stage_rmw<C, H, NX, 0, true, NY, 1, PX, 0, 1, false>(
-        twx, [&](int, int i, int) { return buf[MF_AT(i, NY * PX)]; }, [&](int q, int e) { return fetch((long long)q * H + e); },
-        [&](int q, int e, C v, C r) { emit((long long)q * H + e, v, r); });
+        twx, [&](int q, int, int e) { return buf[MF_AT(x_row<NX>(q) * PX + e, NY * PX)]; },
+        [&](int q, int e) { return fetch((long long)x_row<NX>(q) * H + e); },
+        [&](int q, int e, C v, C r) { emit((long long)x_row<NX>(q) * H + e, v, r); });
   } else {
     if constexpr (sizeof(C) == 8 && RowPlan<H>::NST == 2) {
-      fft2::stage<C, H, NX, 0, true, NY, 1, PX, 0, 1, false>(buf, twx);
+      fft2::stage_io<C, H, NX, 0, true, NY, 1, PX, 0, 1, false>(
+          twx, [&](int q, int, int e) { return buf[MF_AT(x_row<NX>(q) * PX + e, NY * PX)]; },
+          [&](int q, int, int e, C v) { buf[MF_AT(x_row<NX>(q) * PX + e, NY * PX)] = v; });
       __syncthreads();
     }
     constexpr int kAhead = MODE == 3 ? 4 : 1;   // values of r in flight per thread
@@ -640,8 +655,17 @@ struct ZShape {
   typedef typename CT<T>::t C;
   static constexpr int S = S_;
   static constexpr bool E8 = sizeof(C) == 8;
-  static constexpr int ZS = S + ((E8 && S < 16) ? 1 : 0);
-  static constexpr int CP = NZ * ZS + (E8 ? (S == 8 ? 1 : 0) : (S == 4 ? 4 : 0));
+  // FP32: pitches with the fewest shared-memory wavefronts over the stages'
+  // access patterns (counted for every pitch up to 2 S and padding up to 15).
+  // The 24 sequences a warp runs through are three components of eight
+  // columns, so components half of the 16 banks apart (CP = 8 mod 16) and, for
+  // the lengths with a factor three or a radix-16 last stage, unpadded z rows;
+  // per block of eight columns 896 instead of 1152 wavefronts at nz = 128, 448
+  // instead of 576 at 64, 1216 instead of 2240 at 96, 2816 instead of 4608 at
+  // 256 with the former S + 1 and CP = 1 mod 16.
+  static constexpr bool kFlat = NZ == 16 || NZ == 48 || NZ == 96 || NZ == 256;
+  static constexpr int ZS = S + ((E8 && S < 16 && !kFlat) ? (S == 8 && NZ == 32 ? 2 : 1) : 0);
+  static constexpr int CP = NZ * ZS + (E8 ? (S == 8 ? 8 : (S == 4 ? (kFlat && NZ > 16 ? 12 : 4) : 0)) : (S == 4 ? 4 : 0));
   // after the three components: twz (NZ), zk (NZ ints), xiz (NZ reals)
   static constexpr size_t smem() {
     return (size_t)3 * CP * sizeof(C) + (size_t)NZ * sizeof(C) + (size_t)NZ * sizeof(int) +

@@ -238,6 +238,7 @@ struct mf_ctx {
   int predictor = MF_PRED_UNIFORM;  // mf_set_predictor
   HistState keep;                   // the history fields that persist between calls (nprev, t1, ...)
   char* pin = nullptr;              // pinned staging of the history block (cudaMallocHost)
+  char* pin_small = nullptr;        // pinned landing place of scalar blocks and averages (first use allocates it)
   std::vector<HistGraph> hist;      // instantiated history graphs
   cudaStream_t caps[5] = {nullptr, nullptr, nullptr, nullptr, nullptr};   // capture streams, one per nesting level
   long long serial = 0;             // creation number (batched-graph cache key)
@@ -365,11 +366,24 @@ MatArgs mat_args(const mf_ctx* c) {
   return m;
 }
 
-int read_scalars(mf_ctx* c, Scalars* h) {
-  cudaError_t e = cudaMemcpyAsync(h, c->ws + c->osc, sizeof(Scalars), cudaMemcpyDeviceToHost, c->st);
-  if (e != cudaSuccess) return MF_CUDA_ERROR;
-  return cuda_status(cudaStreamSynchronize(c->st));
+// A few device values (at most kSmallBytes) to the host, after everything on
+// the context's stream: through pinned memory, which the copy engine writes
+// in stream order (a copy to pageable memory waits in the driver first).
+constexpr size_t kSmallBytes = 1024;
+static_assert(sizeof(Scalars) <= kSmallBytes, "the scalar block fits");
+int read_small(mf_ctx* c, void* dst, size_t off, size_t bytes) {
+  if (!c->pin_small && cudaMallocHost((void**)&c->pin_small, kSmallBytes) != cudaSuccess) {
+    cudaGetLastError();
+    c->pin_small = nullptr;
+  }
+  void* to = c->pin_small ? (void*)c->pin_small : dst;
+  cudaError_t e = cudaMemcpyAsync(to, c->ws + off, bytes, cudaMemcpyDeviceToHost, c->st);
+  if (e == cudaSuccess) e = cudaStreamSynchronize(c->st);
+  if (e == cudaSuccess && to != dst) memcpy(dst, to, bytes);
+  return cuda_status(e);
 }
+
+int read_scalars(mf_ctx* c, Scalars* h) { return read_small(c, h, c->osc, sizeof(Scalars)); }
 
 int flags_status(int flags) {
   if (flags & MF_FLAG_TIMEOUT) return MF_DEVICE_TIMEOUT;
@@ -1637,12 +1651,7 @@ int mf_residual(mf_ctx* c, const uint8_t* mask, const double* pbar, double* b_de
   double* mean = c->at<double>(c->ores);
   int s = run_residual(c, mask, pbar, b_dev, mean);
   if (s) return s;
-  if (meanP_host) {
-    cudaError_t e = cudaMemcpyAsync(meanP_host, mean, 9 * sizeof(double), cudaMemcpyDeviceToHost, c->st);
-    if (e == cudaSuccess) e = cudaStreamSynchronize(c->st);
-    return cuda_status(e);
-  }
-  return MF_OK;
+  return meanP_host ? read_small(c, meanP_host, c->ores, 9 * sizeof(double)) : MF_OK;
 }
 
 int mf_solve(mf_ctx* c, int nsteps, const uint8_t* mask, const double* target, double tol_newton,
@@ -2153,6 +2162,7 @@ void mf_destroy(mf_ctx* c) {
   for (cudaStream_t s : c->caps)
     if (s) cudaStreamDestroy(s);
   if (c->pin) cudaFreeHost(c->pin);
+  if (c->pin_small) cudaFreeHost(c->pin_small);
   mf_cufft_delete(c->cufft);
   delete c;
 }

@@ -28,7 +28,7 @@ LIB_TRACE = os.path.join(HERE, "libmixfft_trace.so")
 SOURCES = ["transform.cu", "transform2_f32.cu", "transform2_f64.cu", "transformg_f32.cu",
            "transformg_f64.cu", "pointwise.cu", "cg.cu", "history.cu",
            "mixfft.cu", "noalloc.cu", "cufft_path.cu", "adjoint.cu", "transform2_dw.cu",
-           "constitutive_dw.cu", "probe.cu"]
+           "constitutive_dw.cu", "tangent_rows.cu", "probe.cu"]
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 FLAGS = ["-O3", "-lineinfo", "-std=c++17", "-Xcompiler", "-fPIC",
          "-Xptxas", "-v"]

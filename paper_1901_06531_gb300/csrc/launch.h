@@ -31,6 +31,7 @@ cudaError_t launch_k(bool pdl, void (*k)(KArgs...), dim3 g, dim3 b, size_t sm, c
 struct XYArgs {
   int v2;          // 1: fixed-size kernels (transform2*.cu), tables of that layout; 0: any-size (transformg.cuh)
   int split;       // with v2: separate row (x) and column (y) kernels (transform3.cuh)
+  int rows_done;   // with split: the row spectra are in the spectrum buffer already (mf_launch_tangent_rows)
   const int* skip; // if non-null and *skip != 0 the kernel returns at once (finished CG)
   int fin;         // fused (not split) inverse pass with the CG update: finish beta in its last block
   int pdl;         // fused kernels: launch with programmatic dependent launch (see launch_k)
@@ -153,6 +154,12 @@ struct TangentArgs {
 cudaError_t mf_launch_tangent(const void* pin, const void* r, void* pout, void* x, bool f32, int tan,
                               bool cg, const TangentArgs& ta, void* t, long long N, double* partials,
                               int nblk, Scalars* sc, cudaStream_t st, bool fin_alpha = false, bool pdl = false);
+// tangent_rows.cu: the FP32 tangent pass (tan 1, 2; cg with the fused finish of
+// alpha) that leaves the row spectra of t in spec instead of t (split planes;
+// the x-y forward pass then runs with rows_done)
+cudaError_t mf_launch_tangent_rows(const void* pin, const void* r, void* pout, void* x, int tan, bool cg,
+                                   const TangentArgs& ta, void* spec, const XYArgs& a, double* partials, Scalars* sc,
+                                   cudaStream_t st);
 cudaError_t mf_launch_fin_beta(const double* partials, int n, Scalars* sc, cudaStream_t st);
 cudaError_t mf_launch_cg_batch_init(Scalars* sc, int max_its, cudaStream_t st);
 cudaError_t mf_launch_cg_cond(const Scalars* sc, cudaGraphConditionalHandle h, cudaStream_t st, bool pdl = false);

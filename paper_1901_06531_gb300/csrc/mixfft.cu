@@ -471,13 +471,20 @@ int tangent_kind(const mf_ctx* c) {
   return c->model == MF_NEOHOOKE ? 1 : 2;
 }
 
+// FP32 tangent pass fused with the x transform (split planes only).
+bool fuse_rows(const mf_ctx* c) { return c->f32() && c->v2 && c->xy_split; }
+
 // y = G*(K : x) for a device vector x of the inner type.
 int run_matvec(mf_ctx* c, const void* x, void* y, const uint8_t* mask) {
   const ZArgs za = z_args(c, c->f32(), mask, 1.0 / (double)c->N);
-  const XYArgs xa = xy_args(c, c->f32());
-  cudaError_t e = mf_launch_tangent(x, nullptr, nullptr, nullptr, c->f32(), tangent_kind(c), false,
-                                    tangent_args(c), c->ws + c->oAp, c->N, nullptr, c->pw_blocks,
-                                    nullptr, c->st, false, true);
+  XYArgs xa = xy_args(c, c->f32());
+  xa.rows_done = fuse_rows(c) ? 1 : 0;
+  cudaError_t e =
+      xa.rows_done
+          ? mf_launch_tangent_rows(x, nullptr, nullptr, nullptr, tangent_kind(c), false, tangent_args(c),
+                                   c->ws + c->ospec, xa, nullptr, nullptr, c->st)
+          : mf_launch_tangent(x, nullptr, nullptr, nullptr, c->f32(), tangent_kind(c), false, tangent_args(c),
+                              c->ws + c->oAp, c->N, nullptr, c->pw_blocks, nullptr, c->st, false, true);
   if (e == cudaSuccess)
     e = mf_launch_project(c->f32(), c->ws + c->oAp, c->ws + c->ospec, y, 0, nullptr, xa, za, nullptr,
                           c->st);
@@ -541,19 +548,22 @@ cudaError_t capture_cg_body(mf_ctx* c, cudaStream_t cs, cudaGraph_t body, const 
   // predecessor's completion (saves the launch gap: 8 CG-bound 32^3 cells
   // solve in half the time; neutral at 128^3)
   const bool pdl = !xa.split;
+  xa.rows_done = fuse_rows(c) ? 1 : 0;
   const TangentArgs ta = tangent_args(c);
   const int tk = tangent_kind(c);
   const int nplanes = mf_xy_blocks(c->ny, c->nz, c->xy_split != 0);
   cudaError_t e = cudaStreamBeginCaptureToGraph(cs, body, nullptr, nullptr, 0, cudaStreamCaptureModeRelaxed);
   for (int it = 0; it < 2 && e == cudaSuccess; ++it) {
-    e = mf_launch_tangent(pbuf[it], r, pbuf[1 - it], x, f32, tk, true, ta, t, c->N, part, c->pw_blocks, sc,
-                          cs, true, pdl);
+    e = xa.rows_done ? mf_launch_tangent_rows(pbuf[it], r, pbuf[1 - it], x, tk, true, ta, c->ws + c->ospec, xa, part,
+                                              sc, cs)
+                     : mf_launch_tangent(pbuf[it], r, pbuf[1 - it], x, f32, tk, true, ta, t, c->N, part, c->pw_blocks,
+                                         sc, cs, true, pdl);
     if (e == cudaSuccess) e = mf_launch_project(f32, t, c->ws + c->ospec, r, 3, part, xa, za, sc, cs);
     if (e == cudaSuccess && !xa.fin) e = mf_launch_fin_beta(part, nplanes, sc, cs);
   }
   // per iteration: tangent, the transform passes (two more for the split x-y
   // kernels), k_fin_beta unless fused; k_cg_cond once per body
-  c->cg_body_kernels = 2 * (1 + (xa.split ? 5 : 3) + (xa.fin ? 0 : 1)) + 1;
+  c->cg_body_kernels = 2 * (1 + (xa.split ? 5 - xa.rows_done : 3) + (xa.fin ? 0 : 1)) + 1;
   if (e == cudaSuccess) e = mf_launch_cg_cond(sc, h, cs, pdl);
   cudaGraph_t captured = nullptr;
   const cudaError_t e2 = cudaStreamEndCapture(cs, &captured);

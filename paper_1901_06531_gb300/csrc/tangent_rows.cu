@@ -1,6 +1,6 @@
 // Tangent pass and x transform in one kernel, for x-y planes that the separate
 // row and column kernels serve (transform3.cuh, nx = ny = 256): a block takes
-// kRowVoxels consecutive voxels (whole rows), evaluates t = K : p there (with
+// RowVoxels consecutive voxels (whole rows), evaluates t = K : p there (with
 // the CG vector updates of k_tangent inside a solve), keeps the nine
 // components of t in shared memory as half-length complex rows, transforms
 // them and writes the row spectra.  t itself never reaches memory: 72 bytes
@@ -13,11 +13,15 @@
 namespace {
 
 constexpr int kThreads = 256;
-constexpr int kRowVoxels = 512;         // two per thread
+// Voxels per group: two per thread inside a solve, four for the operator alone,
+// which has three of its streams less to load before a group's transform
+// (256^3 operator, neo-Hookean 1455 -> 1444 us, SVK 1521 -> 1487; inside a solve
+// four are slower: 113.1 -> 115.3 ms for 32 SVK iterations at 256^3)
+template <bool CG> struct RowVoxels { static constexpr int value = CG ? 512 : 1024; };
 constexpr int kMaxBlocks = 152 * 4;     // resident at once; each walks over groups of rows
 
-template <int NX> struct RowsShape {
-  static constexpr int H = NX / 2, PX = H + 1, ROWS = kRowVoxels / NX, NSEQ = 9 * ROWS;
+template <int NX, bool CG> struct RowsShape {
+  static constexpr int H = NX / 2, PX = H + 1, ROWS = RowVoxels<CG>::value / NX, NSEQ = 9 * ROWS;
   static constexpr size_t smem() {
     return (size_t)NSEQ * PX * sizeof(float2) + (size_t)NX * sizeof(float2) + (size_t)H * sizeof(int);
   }
@@ -30,7 +34,8 @@ __global__ void __launch_bounds__(kThreads, 4)
                    const float2* __restrict__ gtw, const int* __restrict__ gpos, double* __restrict__ partials,
                    Scalars* sc) {
   typedef float2 C;
-  typedef RowsShape<NX> Sh;
+  typedef RowsShape<NX, CG> Sh;
+  constexpr int kRowVoxels = RowVoxels<CG>::value;
   constexpr int H = Sh::H, PX = Sh::PX, ROWS = Sh::ROWS, NSEQ = Sh::NSEQ, NY = NX;
   static_assert(kRowVoxels % NX == 0 && NY % ROWS == 0, "whole rows, groups within a plane");
   extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -128,8 +133,8 @@ __global__ void __launch_bounds__(kThreads, 4)
 template <int NX, int TAN, bool CG>
 cudaError_t launch_rows(const float* pin, const float* r, float* pout, float* x, const TangentArgs& ta, void* spec,
                         const XYArgs& a, double* partials, Scalars* sc, cudaStream_t st) {
-  const size_t sm = RowsShape<NX>::smem();
-  const long long groups = a.N / kRowVoxels;
+  const size_t sm = RowsShape<NX, CG>::smem();
+  const long long groups = a.N / RowVoxels<CG>::value;
   const int grid = (int)(groups < kMaxBlocks ? groups : kMaxBlocks);
   ++g_mf_launches;
   k_tangent_rows<NX, TAN, CG><<<grid, kThreads, sm, st>>>(pin, r, pout, x, ta, (float2*)spec, a.nz, a.N,

@@ -60,12 +60,14 @@ template <typename T, int NX> __host__ __device__ constexpr int xy_min_blocks() 
 // 128-point transform and two in its radix-8 stage (3 x S x 128/R)
 __host__ __device__ constexpr int z_threads(int S) { return 24 * S; }
 // resident z-pass blocks per SM the register allocation is held to: five
-// blocks of 192 threads for the FP32 operator pass (S = 8, MODE 0), three for
+// blocks of 192 threads for the FP32 operator pass (S = 8, MODE 0; four at nz =
+// 256, where shared memory holds no more and 80 registers take the spills out of
+// its radix-16 stages: 256^3 392 -> 380 us), three for
 // the double-word residual (112 registers instead of 138: 128^3 residual 698
 // -> 686 us), else what the compiler chooses
-template <typename T> __host__ __device__ constexpr int z_min_blocks(int S, int mode) {
+template <typename T> __host__ __device__ constexpr int z_min_blocks(int S, int mode, int nz) {
   if (S == 8 && std::is_same<T, dw>::value) return 3;
-  return (sizeof(typename CT<T>::t) == 8 && S == 8 && mode == 0) ? 5 : 1;
+  return (sizeof(typename CT<T>::t) == 8 && S == 8 && mode == 0) ? (nz == 256 ? 4 : 5) : 1;
 }
 
 // Asynchronous global -> shared copies of one complex element (8 or 16
@@ -678,7 +680,7 @@ struct ZShape {
 // null frequency, records the null-frequency coefficient / N in a.mean_out).
 // Grid: 3 row groups x (ncol / S) column tiles.
 template <typename T, int NZ, int MODE, int S_>
-__global__ void __launch_bounds__(z_threads(S_), z_min_blocks<T>(S_, MODE)) k_zp(typename CT<T>::t* __restrict__ spec, ZArgs a) {
+__global__ void __launch_bounds__(z_threads(S_), z_min_blocks<T>(S_, MODE, NZ)) k_zp(typename CT<T>::t* __restrict__ spec, ZArgs a) {
   typedef ZShape<T, NZ, S_> Sh;
   constexpr int kZThreads = z_threads(S_);
   typedef typename CT<T>::t C;
@@ -698,7 +700,7 @@ __global__ void __launch_bounds__(z_threads(S_), z_min_blocks<T>(S_, MODE)) k_zp
     const int kz = a.zk[i];
     zk[i] = kz;
     const int kzs = (2 * kz < NZ) ? kz : kz - NZ;
-    if constexpr (!Sh::E8) xiz[i] = (T)kzs * ((T)1 / (T)NZ);
+    if constexpr (!Sh::E8 || RL > 8) xiz[i] = (T)kzs * ((T)1 / (T)NZ);
   }
   pdl_wait();
   __shared__ int s_stop;   // tested after the first barrier (see k_xyf)
@@ -825,7 +827,8 @@ __global__ void __launch_bounds__(z_threads(S_), z_min_blocks<T>(S_, MODE)) k_zp
     // passes over shared memory.  So they are in FP32 where the last stage is
     // radix 16: for nz = 16, one stage, registers left eight threads a block
     // with all the work (14 us a launch); for nz = 256 three butterflies of 16
-    // do not fit the 64 registers of the tile's occupancy (0.9 KB of spills)
+    // do not fit the registers of the occupancy that shared memory allows (80;
+    // 0.9 KB of spills at 64)
     if constexpr (NST == 1) {
       for (int idx = threadIdx.x; idx < 3 * NZ * S; idx += kZThreads) {
         const int s2 = idx % S, cz = idx / S, cl = cz / NZ, z = cz - cl * NZ;
@@ -836,39 +839,34 @@ __global__ void __launch_bounds__(z_threads(S_), z_min_blocks<T>(S_, MODE)) k_zp
     }
     fft2::stage<C, NZ, NZ, NST - 1, false, 3 * S, S, CP, 1, ZS, true>(buf, twz);
     __syncthreads();
-    if constexpr (Sh::E8) {
-      for (int idx = threadIdx.x; idx < NZ * S; idx += kZThreads) {
-        const int s2 = idx % S, z = idx / S;
-        C* e = buf + z * ZS + s2;
+    // a thread keeps one column: xi_x, xi_y and the sum of their squares are
+    // taken once, xi_z from the table (in 16-byte types every product and
+    // conversion of gstar counts: 64^3 FP64 operator 368.7 -> 361.3 us; the
+    // values are the same)
+    static_assert(kZThreads % S == 0, "one column per thread");
+    const int s2 = threadIdx.x % S, col = col0 + s2;
+    const int row = col / H, slot = col - (col / H) * H;
+    const int kx = a.xk[slot], ky = a.yk[row];
+    const T xi0 = (T)kx * rnx, xi1 = (T)((2 * ky < a.ny) ? ky : ky - a.ny) * rny;
+    const T xi01 = xi0 * xi0 + xi1 * xi1;
+    for (int z = threadIdx.x / S; z < NZ; z += kZThreads / S) {
+      C* e = buf + z * ZS + s2;
+      const int kz = zk[z];
+      if ((2 * ky == a.ny) || ((NZ % 2 == 0) && (2 * kz == NZ)) || (kx == 0 && ky == 0 && kz == 0)) {
         gstar(s2, z, e[0], e[CP], e[2 * CP]);
-      }
-    } else {
-      // a thread keeps one column: xi_x, xi_y and the sum of their squares are
-      // taken once, xi_z from the table (in 16-byte types every product and
-      // conversion of gstar counts: 64^3 FP64 operator 368.7 -> 361.3 us; the
-      // values are the same)
-      static_assert(kZThreads % S == 0, "one column per thread");
-      const int s2 = threadIdx.x % S, col = col0 + s2;
-      const int row = col / H, slot = col - (col / H) * H;
-      const int kx = a.xk[slot], ky = a.yk[row];
-      const T xi0 = (T)kx * rnx, xi1 = (T)((2 * ky < a.ny) ? ky : ky - a.ny) * rny;
-      const T xi01 = xi0 * xi0 + xi1 * xi1;
-      for (int z = threadIdx.x / S; z < NZ; z += kZThreads / S) {
-        C* e = buf + z * ZS + s2;
-        const int kz = zk[z];
-        if ((2 * ky == a.ny) || ((NZ % 2 == 0) && (2 * kz == NZ)) || (kx == 0 && ky == 0 && kz == 0)) {
-          gstar(s2, z, e[0], e[CP], e[2 * CP]);
-        } else {
-          const T xi2 = xiz[z];
-          const T inv = scale / (xi01 + xi2 * xi2);
-          const C v0 = e[0], v1 = e[CP], v2 = e[2 * CP];
-          C q;
-          q.x = (v0.x * xi0 + v1.x * xi1 + v2.x * xi2) * inv;
-          q.y = (v0.y * xi0 + v1.y * xi1 + v2.y * xi2) * inv;
-          e[0] = cmake(q.x * xi0, q.y * xi0);
-          e[CP] = cmake(q.x * xi1, q.y * xi1);
-          e[2 * CP] = cmake(q.x * xi2, q.y * xi2);
-        }
+      } else {
+        const T xi2 = xiz[z];
+        const T den = xi01 + xi2 * xi2;
+        T inv;
+        if constexpr (sizeof(T) == 4) inv = scale * __frcp_rn(den);
+        else inv = scale / den;
+        const C v0 = e[0], v1 = e[CP], v2 = e[2 * CP];
+        C q;
+        q.x = (v0.x * xi0 + v1.x * xi1 + v2.x * xi2) * inv;
+        q.y = (v0.y * xi0 + v1.y * xi1 + v2.y * xi2) * inv;
+        e[0] = cmake(q.x * xi0, q.y * xi0);
+        e[CP] = cmake(q.x * xi1, q.y * xi1);
+        e[2 * CP] = cmake(q.x * xi2, q.y * xi2);
       }
     }
     __syncthreads();

@@ -78,7 +78,7 @@ def measured_peaks():
 
 # source files each timed kernel is compiled from
 KERNEL_SOURCES = {
-    "tangent_cg": ("cg.cu", "common.cuh", "launch.h"),
+    "tangent_cg": ("cg.cu", "tangent.cuh", "common.cuh", "launch.h"),
     "xy_forward": ("transform2.cuh", "transform2c.cuh", "transform2_impl.cuh", "fft2.cuh", "common.cuh", "dw.cuh",
                    "launch.h"),
     "zpass_projection": ("transform2.cuh", "transform2_impl.cuh", "fft2.cuh", "common.cuh", "dw.cuh", "launch.h"),

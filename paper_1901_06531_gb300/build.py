@@ -16,7 +16,7 @@ HERE = os.path.dirname(os.path.abspath(__file__))
 CSRC = os.path.join(HERE, "csrc")
 BUILD = os.path.join(HERE, "_build")
 LIB = os.path.join(HERE, "libmixfft.so")
-# debug build: every shared- and global-memory index of the generic and
+# debug build: every shared- and global-memory index of the any-size and
 # fixed-size transform kernels and the tangent pass checked (MF_DEBUG, see
 # common.cuh)
 BUILD_DEBUG = os.path.join(HERE, "_build_debug")

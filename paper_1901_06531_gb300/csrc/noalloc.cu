@@ -99,7 +99,7 @@ extern "C" int mf_residual_noalloc(int nx, int ny, int nz, const double* P_dev, 
   if (e != cudaSuccess) return MF_CUDA_ERROR;
 
   XYArgs xa;
-  memset(&xa, 0, sizeof(xa));   // persist, flags and the rest unused by the generic kernels: zero
+  memset(&xa, 0, sizeof(xa));   // persist, flags and the rest unused by the any-size kernels: zero
   xa.v2 = 0;
   xa.split = 0;
   xa.skip = nullptr;

@@ -378,6 +378,8 @@ __global__ void __launch_bounds__(xy_threads<T, NX>(), xy_min_blocks<T, NX>()) k
     }
   }
   __syncthreads();
+  // one-stage row transforms (NX = 16, 32) meet their first barrier here
+  if (s_stop) return;
   // y: H columns of NY samples, stride PX; the last stage stores the
   // spectrum rows (consecutive threads take consecutive columns)
   C* dst = spec + ((long long)c * nz + z) * NY * H;

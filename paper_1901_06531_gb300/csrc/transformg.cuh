@@ -27,6 +27,8 @@
 // 125.2 -> 67.8 us, stress and residual in FP64 on 48 x 36 x 18 184 -> 147 us.
 #pragma once
 
+#include <atomic>
+
 #include "launch.h"
 
 namespace trg {
@@ -504,11 +506,20 @@ inline int pick_threads(int regs, size_t smem, int blocks, int work, int most) {
   return best;
 }
 
+// Registers a thread of kernel K, asked for once (the same on every device
+// this code runs on); a query that fails is asked again at the next launch.
 template <auto K> int regs_of() {
-  static const int n = [] {
+  static std::atomic<int> known{0};
+  int n = known.load(std::memory_order_relaxed);
+  if (n == 0) {
     cudaFuncAttributes at;
-    return cudaFuncGetAttributes(&at, K) == cudaSuccess ? at.numRegs : 128;
-  }();
+    if (cudaFuncGetAttributes(&at, K) != cudaSuccess) {
+      cudaGetLastError();
+      return 128;
+    }
+    n = at.numRegs;
+    known.store(n, std::memory_order_relaxed);
+  }
   return n;
 }
 
@@ -524,22 +535,28 @@ size_t xy_smem(const XYArgs& a) {
   return (size_t)(a.ny / 2) * pitch(a.nx) * sizeof(C) + (size_t)(a.nx + a.ny) * sizeof(C) + (size_t)a.nx * sizeof(int);
 }
 
-// The shared-memory opt-in, once per kernel and process (one process drives
-// one device), at the most a plane of any admissible size takes.
-constexpr size_t kSmemMax = 226 * 1024;
+// The shared-memory opt-in, at every launch that needs one: it belongs to a
+// device, and contexts on several devices of a process, and the residual
+// without a context on whichever device its caller has current, run these
+// kernels.
+// Always at the most a plane of any admissible size takes, so that host
+// threads launching different sizes set the same value.  Launches that stay
+// within the default 48 KB with the kernels' static part (below 1 KB) need
+// none: planes up to 72 x 72 in FP64, 108 x 96 in FP32.
+constexpr size_t kSmemMax = 226 * 1024, kSmemDefault = 47 * 1024;
 template <auto K>
-cudaError_t smem_once() {
-  static const cudaError_t e = cudaFuncSetAttribute(K, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmemMax);
-  return e;
+cudaError_t smem_opt_in(size_t sm) {
+  if (sm <= kSmemDefault) return cudaSuccess;
+  if (sm > kSmemMax) return cudaErrorInvalidValue;
+  return cudaFuncSetAttribute(K, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmemMax);
 }
 
 template <typename T>
 cudaError_t xyf(const void* in, void* spec, const XYArgs& a, cudaStream_t st) {
   typedef typename CT<T>::t C;
-  const cudaError_t e = smem_once<k_xyf<T>>();
-  if (e != cudaSuccess) return e;
   const size_t sm = xy_smem<T>(a);
-  if (sm > kSmemMax) return cudaErrorInvalidValue;
+  const cudaError_t e = smem_opt_in<k_xyf<T>>(sm);
+  if (e != cudaSuccess) return e;
   ++g_mf_launches;
   const int t = pick_threads(regs_of<k_xyf<T>>(), sm, 9 * a.nz, xy_work(a), 512);
   return launch_k(a.pdl != 0, k_xyf<T>, dim3(9 * a.nz), dim3(t), sm, st, (const T*)in, (C*)spec, a);
@@ -548,10 +565,9 @@ cudaError_t xyf(const void* in, void* spec, const XYArgs& a, cudaStream_t st) {
 template <typename T, int MODE>
 cudaError_t xyi_m(const void* spec, void* out, double* partials, const XYArgs& a, const Scalars* sc, cudaStream_t st) {
   typedef typename CT<T>::t C;
-  const cudaError_t e = smem_once<k_xyi<T, MODE>>();
-  if (e != cudaSuccess) return e;
   const size_t sm = xy_smem<T>(a);
-  if (sm > kSmemMax) return cudaErrorInvalidValue;
+  const cudaError_t e = smem_opt_in<k_xyi<T, MODE>>(sm);
+  if (e != cudaSuccess) return e;
   ++g_mf_launches;
   const int t = pick_threads(regs_of<k_xyi<T, MODE>>(), sm, 9 * a.nz, xy_work(a), 512);
   return launch_k(a.pdl != 0, k_xyi<T, MODE>, dim3(9 * a.nz), dim3(t), sm, st, (const C*)spec, (T*)out, partials, a,
@@ -567,10 +583,9 @@ cudaError_t xyi(int mode, const void* spec, void* out, double* partials, const X
 template <typename T, int MODE, int S>
 cudaError_t zp_s(void* spec, ZArgs a, cudaStream_t st) {
   typedef typename CT<T>::t C;
-  const cudaError_t e = smem_once<k_zp<T, MODE, S>>();
-  if (e != cudaSuccess) return e;
   const size_t sm = (size_t)3 * ZPad<T>::cp(a.nz, S) * sizeof(C) + (size_t)a.nz * (sizeof(C) + sizeof(T) + sizeof(int));
-  if (sm > kSmemMax) return cudaErrorInvalidValue;
+  const cudaError_t e = smem_opt_in<k_zp<T, MODE, S>>(sm);
+  if (e != cudaSuccess) return e;
   const int ncol = a.ny * (a.nx / 2);
   a.dseq = fast_div(3 * S);
   const int blocks = 3 * ((ncol + S - 1) / S);

@@ -230,7 +230,9 @@ int mf_residual_noalloc(int nx, int ny, int nz, const double* P_dev, const uint8
  * memset of the 9N-double residual buffer): [0] the tangent pass (direction
  * and solution updates, K:p, p.Kp), [1] the x-y forward transform, [2] the
  * z-pass with G-hat-star, [3] the x-y inverse transform with the residual
- * update.  Operands are the context's CG vectors; needs the operator of the
+ * update.  FP32-inner contexts with separate row and column kernels
+ * (mf_set_xy_split) run the row transform inside the tangent pass: there [0]
+ * is both and [1] the column transform alone.  Operands are the context's CG vectors; needs the operator of the
  * last mf_constitutive.  graph 0: events around every launch (the time
  * includes the launch's own start-up on the device); graph 1: the reps
  * (flush, launch) pairs run as one CUDA graph, events around the graph, minus

@@ -1806,7 +1806,8 @@ int mf_time_kernels(mf_ctx* c, const uint8_t* mask, int reps, int graph, float* 
   if (!operator_ready(c)) return MF_INVALID_ARG;
   const bool f32 = c->f32();
   const ZArgs za = z_args(c, f32, mask, 1.0 / (double)c->N);
-  const XYArgs xa = xy_args(c, f32);
+  XYArgs xa = xy_args(c, f32);
+  xa.rows_done = fuse_rows(c) ? 1 : 0;   // as inside a solve
   const TangentArgs ta = tangent_args(c);
   Scalars* sc = c->at<Scalars>(c->osc);
   double* part = c->at<double>(c->opart);
@@ -1823,10 +1824,20 @@ int mf_time_kernels(mf_ctx* c, const uint8_t* mask, int reps, int graph, float* 
   cudaEvent_t e0, e1;
   if (e != cudaSuccess || cudaEventCreate(&e0) != cudaSuccess) return MF_CUDA_ERROR;
   if (cudaEventCreate(&e1) != cudaSuccess) { cudaEventDestroy(e0); return MF_CUDA_ERROR; }
+  // the fused tangent and row pass sets alpha itself, and the stop flag where
+  // the vectors' curvature is none: cleared before each launch
+  auto rearm = [&](cudaStream_t s) {
+    cudaError_t ee = cudaMemsetAsync(&sc->stop, 0, sizeof(sc->stop), s);
+    return ee == cudaSuccess ? cudaMemsetAsync(&sc->flags, 0, sizeof(sc->flags), s) : ee;
+  };
   auto flush = [&](cudaStream_t s, int r) {   // L2 flush: a memset larger than L2
-    return cudaMemsetAsync(c->ws + c->ob, r & 0xff, 9 * c->N * sizeof(double), s);
+    const cudaError_t ee = cudaMemsetAsync(c->ws + c->ob, r & 0xff, 9 * c->N * sizeof(double), s);
+    return ee == cudaSuccess && xa.rows_done ? rearm(s) : ee;
   };
   auto kernel = [&](cudaStream_t s, int which) {
+    if (which == 0 && xa.rows_done)
+      return mf_launch_tangent_rows(c->ws + c->op, c->ws + c->or_, c->ws + c->op2, c->ws + c->ox, tangent_kind(c), true,
+                                    ta, c->ws + c->ospec, xa, part, sc, s);
     if (which == 0)
       return mf_launch_tangent(c->ws + c->op, c->ws + c->or_, c->ws + c->op2, c->ws + c->ox, f32, tangent_kind(c),
                                true, ta, c->ws + c->oAp, c->N, part, c->pw_blocks, sc, s);
@@ -1861,6 +1872,11 @@ int mf_time_kernels(mf_ctx* c, const uint8_t* mask, int reps, int graph, float* 
   float base = 0.f;
   if (graph) e = graph_ms(-1, &base);
   for (int which = 0; which < 4 && e == cudaSuccess; ++which) {
+    // the column pass alone, in place and unscaled, would grow what it is
+    // repeated on
+    if (which == 1 && xa.rows_done)
+      e = cudaMemsetAsync(c->ws + c->ospec, 0, 9 * c->N * sizeof(float), c->st);
+    if (e != cudaSuccess) break;
     if (graph) {
       float ms = 0.f;
       e = graph_ms(which, &ms);
@@ -1880,6 +1896,7 @@ int mf_time_kernels(mf_ctx* c, const uint8_t* mask, int reps, int graph, float* 
     }
     ms_out[which] = (float)(tot / reps);
   }
+  if (e == cudaSuccess && xa.rows_done) e = rearm(c->st);
   cudaEventDestroy(e0);
   cudaEventDestroy(e1);
   if (e != cudaSuccess) cudaGetLastError();

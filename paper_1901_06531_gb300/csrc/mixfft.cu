@@ -282,10 +282,16 @@ namespace {
 
 // Whether a context whose grid has fixed-size kernels uses them.  FP32-inner
 // contexts do.  Plain FP64 is bound by the FP64 pipe, or on small cells by how
-// many threads share its chains: per CG iteration the any-size kernels take
-// 44, 74, 190 and 1503 us against 58, 95, 256 and 1562 us on 16^3, 32^3, 48^3
-// and 96^3, but 474 against 430 us on 64^3 (8 x 8 stages), so planes of 64^2,
-// 128^2 and 256^2 stay with the fixed-size ones.
+// many threads share its chains.  us of an operator application / a CG
+// iteration, any-size against fixed-size kernels: 16^3 29/37 against 39/48,
+// 32^3 56/67 (55/67), 48^3 154/176 (195/218), 96^3 1350/1427 (1347/1435); flat
+// boxes 32 x 32 x 16 37/47 (46/55), 48 x 48 x 16 68/79 (68/80), 96 x 96 x 16
+// 221/250 (238/266); long ones 16 x 16 x 256 161/180 (187/219), 32 x 32 x 128
+// 192/219 (190/221), 48 x 48 x 128 420/464 (448/495), 96 x 96 x 128 1772/1869
+// (1748/1862).  On planes of 64^2 and 128^2 (8 x 8 and 16 x 8 stages) the
+// fixed-size ones win: 64^3 400/445 against 356/404, 64 x 64 x 16 105/119
+// (101/117), 64 x 64 x 256 1620/1717 (1491/1596), 128 x 128 x 32 784/840
+// (741/802); 256^2 has no other.
 int use_fixed_size(const mf_ctx* c) {
   if (!c->v2_ok) return 0;
   return (c->f32() || c->nx == 64 || c->nx == 128 || c->nx == 256) ? 1 : 0;

@@ -59,9 +59,6 @@ __device__ __forceinline__ long long mf_dbg_check(long long i, long long n, int 
 // once.  (No kernel here signals its dependents early: measured on the 128^3
 // cell, dependents resident during the predecessor's last wave slowed it.)
 __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
-// Lets the dependent grid be scheduled once every block of this one has
-// issued it or exited.
-__device__ __forceinline__ void pdl_trigger() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 
 // Grid of a grid-stride elementwise pass over n items with `threads` per
 // block: one item per thread for small passes, at most 8 blocks per SM (152

@@ -156,12 +156,18 @@ cudaError_t xyi_m(const void* spec, void* out, double* partials, const XYArgs& a
       default: return cudaErrorInvalidValue;
     }
   }
+  // the CG update in FP64: on planes of 64 and 128 squared only (plain FP64
+  // contexts use the any-size kernels on the others)
+  if constexpr (!(std::is_same<T, double>::value && MODE == 3)) {
+    switch (a.nx) {
+      case 16: return launch_xyi<T, 16, MODE>(spec, o, partials, a, sc, st);
+      case 32: return launch_xyi<T, 32, MODE>(spec, o, partials, a, sc, st);
+      case 48: return launch_xyi<T, 48, MODE>(spec, o, partials, a, sc, st);
+      case 96: return launch_xyi<T, 96, MODE>(spec, o, partials, a, sc, st);
+    }
+  }
   switch (a.nx) {
-    case 16: return launch_xyi<T, 16, MODE>(spec, o, partials, a, sc, st);
-    case 32: return launch_xyi<T, 32, MODE>(spec, o, partials, a, sc, st);
-    case 48: return launch_xyi<T, 48, MODE>(spec, o, partials, a, sc, st);
     case 64: return launch_xyi<T, 64, MODE>(spec, o, partials, a, sc, st);
-    case 96: return launch_xyi<T, 96, MODE>(spec, o, partials, a, sc, st);
     case 128: return launch_xyi<T, 128, MODE>(spec, o, partials, a, sc, st);
     default: return cudaErrorInvalidValue;
   }

@@ -90,12 +90,16 @@ int mf_bind_workspace(mf_ctx* ctx, void* dev, size_t bytes);
  *          the stiffness of phase p is C'_ijkl = R_ia R_jb R_kc R_ld C_abcd;
  *   scale  host, N doubles multiplying P and K per voxel, or NULL.
  * Copies are enqueued on the stream; the host arrays may be reused on return.
- * Resets F to the identity. */
+ * Resets F to the identity (as mf_set_F with NULL). */
 int mf_set_material(mf_ctx* ctx, int model, int nphase, const double* params,
                     const double* rot, const int32_t* phase, const double* scale);
 
-/* Set the deformation-gradient field from host memory (9N doubles) or, with
- * F_host NULL, to the identity everywhere. */
+/* Set the deformation-gradient field from host memory (9N doubles; the call
+ * waits for the copy) or, with F_host NULL, to the identity everywhere: then
+ * the field is written by the device, ordered on the context's stream, and
+ * the call does not wait for it (no host synchronisation, like mf_load_F; a
+ * device error of work still queued is reported by a later call that waits,
+ * mf_sync among them). */
 int mf_set_F(mf_ctx* ctx, const double* F_host);
 
 /* Run a load history (Sec. 2.3; Sec. 4 stopping rules).

@@ -217,11 +217,8 @@ int mf_residual(mf_ctx* ctx, const uint8_t* mask, const double* pbar, double* b_
  * All other memory -- the half spectrum, index and twiddle tables, reduction
  * partials -- lives in one file-scope static device array of 18,958,592
  * bytes (18.1 MiB) that every GPU loading the library holds until the
- * process exits.  No cudaMalloc or cudaFree is called.  The first call on a
- * device looks up the array's device address (cudaGetSymbolAddress, with that
- * device current) and caches it for the process; make that first call
- * outside any stream capture.  The cached address does not survive a reset
- * of the device (cudaDeviceReset): do not call this entry point after one.
+ * process exits.  No cudaMalloc or cudaFree is called.  Every call looks up
+ * the array's address on the current device (cudaGetSymbolAddress).
  * stream must belong to the current device (MF_INVALID_ARG otherwise).  All
  * calls share the one array and each call overwrites it, so calls that may
  * overlap on the GPU (different streams, or different host threads) race:

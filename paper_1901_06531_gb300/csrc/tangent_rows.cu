@@ -6,7 +6,9 @@
 // them and writes the row spectra.  t itself never reaches memory: 72 bytes
 // per voxel and application less than a tangent pass and a row pass (the
 // operator on a 256^3 cell moved 472 bytes per voxel and is bound by HBM:
-// 1584 -> 1454 us).  Same arithmetic in the same order, so the same bits.
+// 1584 -> 1444 us).  t and its row spectra have the bits of those two; inside a
+// solve p.t is summed over other groups of voxels, so that its last bits (and
+// through alpha now and then an FP32 rounding) are its own.
 #include "tangent.cuh"
 #include "transform3.cuh"
 

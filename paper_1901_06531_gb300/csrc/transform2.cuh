@@ -42,7 +42,8 @@ constexpr int kThreads = 256;
 // threads; planes up to 64 x 64 run three blocks of 256, of 96 x 96 two of
 // 512, whose barriers and load phases overlap (double-word residual against
 // one block of 512: 32^3 31 -> 23 us, 48^3 69 -> 49, 64^3 94 -> 80, 96^3 341
-// -> 310).  FP32 128 x 128 planes (66 KB) run two blocks of 512 threads per
+// -> 310; the 64 registers a thread that 96 x 96 leaves make its kernels spill
+// 220 to 310 bytes, which takes part of that gain back).  FP32 128 x 128 planes (66 KB) run two blocks of 512 threads per
 // SM at 64 registers a thread (about 1% faster than three blocks of 256 on
 // the GB300), other FP32 planes blocks of 256
 constexpr int kXY128Threads = 512;

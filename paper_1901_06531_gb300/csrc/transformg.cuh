@@ -24,7 +24,7 @@
 // passes and indices, in FP32, and the FP64 pipe in FP64.  Against one stage
 // per pass with hardware divisions, whole planes staged before and after, and
 // all nine components in one z-pass block: FP32 operator on 108 x 72 x 54
-// 125.2 -> 67.8 us, stress and residual in FP64 on 48 x 36 x 18 184 -> 147 us.
+// 125 -> 52 us, stress and residual in FP64 on 48 x 36 x 18 184 -> 134 us.
 #pragma once
 
 #include <atomic>

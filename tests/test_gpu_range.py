@@ -40,3 +40,20 @@ def test_small_units_take_the_same_course(shape):
     (g0, i0), (g1, i1) = got
     assert i0 > 10 and abs(i1 - i0) <= 1
     assert np.max(np.abs(g1 - g0)) <= 1e-5 * np.max(np.abs(g0))
+
+
+def test_solve_on_a_larger_grid_against_fp64():
+    """Partial sums of several hundred planes: the FP32-inner solve ends within
+    its field tolerance of 1e-8 of the plain FP64 one."""
+    mf = lib()
+    nx, ny, nz = 72, 54, 36
+    ph, params = neohooke_two_phase((nz, ny, nx), 5)
+    m, t = inputs.fix_rotation(*inputs.history_uniaxial_stress_ramp(2, 0.05))
+    got = []
+    for prec in (mf.MF_FP64, mf.MF_FP32_INNER):
+        ctx = mf.Context(nx, ny, nz, prec)
+        ctx.set_material(mf.MF_NEOHOOKE, params, ph)
+        out = ctx.solve(m, t, 1e-10, 1e-12, cg_rel=1e-4)
+        got.append((ctx.get_fields()[0], out["Fbar"]))
+    assert np.max(np.abs(got[1][0] - got[0][0])) < 1e-8
+    assert np.max(np.abs(got[1][1] - got[0][1])) < 1e-9

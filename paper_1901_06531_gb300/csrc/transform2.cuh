@@ -320,8 +320,16 @@ __global__ void __launch_bounds__(xy_threads<T, NX>(), xy_min_blocks<T, NX>()) k
   // queue) and tested after the first barrier behind the plane's loads
   // (nothing is written before), and the first stage reads its twiddles from
   // global memory: the loads wait neither for the flag nor for the tables
+  // (with one x stage thread 0 hands the flag on after its butterflies: its
+  // warp would hold back their loads until the flag is there, 0.2 us of the
+  // 3 us that a 32 x 32 plane takes)
+  constexpr bool kOneStage = sizeof(C) == 8 && RowPlan<H>::NST == 1;
   __shared__ int s_stop;
-  if (threadIdx.x == 0) s_stop = skip ? *(volatile const int*)skip : 0;
+  int stop = 0;
+  if (threadIdx.x == 0) {
+    stop = skip ? *(volatile const int*)skip : 0;
+    if (!kOneStage) s_stop = stop;
+  }
   const int c = blockIdx.x % 9, z = blockIdx.x / 9;
   const CI* src = reinterpret_cast<const CI*>(in + c * N + (long long)z * NY * NX);
   // row y, sample j (the real values 2j, 2j+1 as one complex sample)
@@ -349,6 +357,7 @@ __global__ void __launch_bounds__(xy_threads<T, NX>(), xy_min_blocks<T, NX>()) k
       x_last_split<T, NX, TPB>(buf, twx, [&](int y, int pos) { return buf[MF_AT(y * PX + pos, NY * PX)]; });
     } else {
       x_last_split<T, NX, TPB>(buf, gtw, gload);
+      if (threadIdx.x == 0) s_stop = stop;
     }
   } else {
     // 16-byte types (FP64, double word) are arithmetic bound: the plane is
@@ -381,7 +390,7 @@ __global__ void __launch_bounds__(xy_threads<T, NX>(), xy_min_blocks<T, NX>()) k
     }
   }
   __syncthreads();
-  // one-stage row transforms (NX = 16, 32) meet their first barrier here
+  // planes of one x stage (NX = 16, 32) meet their first barrier here
   if (s_stop) return;
   // y: H columns of NY samples, stride PX; the last stage stores the
   // spectrum rows (consecutive threads take consecutive columns)

@@ -63,11 +63,11 @@ __host__ __device__ constexpr int z_threads(int S) { return 24 * S; }
 // resident z-pass blocks per SM the register allocation is held to: five
 // blocks of 192 threads for the FP32 operator pass (S = 8, MODE 0; four at nz =
 // 256, where shared memory holds no more and 80 registers take the spills out of
-// its radix-16 stages: 256^3 392 -> 380 us), three for
-// the double-word residual (112 registers instead of 138: 128^3 residual 698
-// -> 686 us; two at nz = 256, again what shared memory holds: at three its 96
-// registers spill without a block more, 64 x 64 x 256 residual 334 -> 326 us,
-// 128 x 128 x 256 1440 -> 1402 us), else what the compiler chooses
+// its radix-16 stages: 256^3 392 -> 380 us), three for the double-word residual
+// (at nz = 128 96 registers instead of 136: residual 698 -> 686 us; two at nz =
+// 256, again what shared memory holds: held to three its 96 registers spill
+// without a block more, 64 x 64 x 256 residual 334 us against 327, 128 x 128 x
+// 256 1438 against 1404), else what the compiler chooses
 template <typename T> __host__ __device__ constexpr int z_min_blocks(int S, int mode, int nz) {
   if (S == 8 && std::is_same<T, dw>::value) return nz == 256 ? 2 : 3;
   return (sizeof(typename CT<T>::t) == 8 && S == 8 && mode == 0) ? (nz == 256 ? 4 : 5) : 1;

@@ -130,7 +130,8 @@ __device__ __forceinline__ void load_tables(C* twx, C* twy, int* posx, const XYA
 }
 
 // Forward x-y transform of one (c, z) plane per block.
-// Registers: 64 a thread in FP32 (two blocks of 512 an SM), 128 in FP64.
+// Registers: 64 a thread in FP32 (two blocks of 512 an SM; the inverse pass
+// spills 80 to 220 bytes for them), 128 in FP64.
 template <typename T> __host__ __device__ constexpr int xy_min_blocks() { return sizeof(T) == 4 ? 2 : 1; }
 
 template <typename T>
